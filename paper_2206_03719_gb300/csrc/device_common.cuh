@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "dfloat.cuh"
+#include "forward_f64.h"
 #include "quantile_f32.h"
 #include "quantile_f64.h"
 
@@ -139,28 +140,77 @@ __device__ __forceinline__ double norm_quantile_f64(double u, double omu) {
   return x * r;
 }
 
+// Tables of a working precision's draws and steps, staged in shared memory by
+// the kernels that step paths (the index differs from lane to lane): double
+// the quantile segments and powers of two of forward_f64.h, float pairs those
+// of df_math.cuh, single precision none.
+struct DfTables;
+struct NoTables {};
+template <typename Real> struct TabOf { using type = NoTables; };
+template <> struct TabOf<double> { using type = F64Tables; };
+template <> struct TabOf<df> { using type = DfTables; };
+template <typename Real> using Tab = typename TabOf<Real>::type;
+
 // Random inputs of one path step from one Philox block: the uniform U_V,
 // 1 - U_V (exact in both grids), Z_V = Phi^-1(U_V) and Z_X.  The float-pair
-// specialisation is in df_math.cuh and uses the tables t stages in shared
-// memory; the others ignore t.
-struct DfTables;
+// specialisation is in df_math.cuh.
 template <typename Real> struct Draw;
 template <> struct Draw<double> {
+  // (m + 1/2) 2^-52, m the top 52 bits of (hi:lo), exact as in uniform52, by
+  // one FP64 subtraction: the integer-to-double conversion runs on the FP64
+  // pipe as well (15 clocks a warp) and needs two operations after it
+  __device__ __forceinline__ static double grid_point(uint32_t hi, uint32_t lo) {
+    return __hiloint2double((int)(0x3ff00000u | (hi >> 12)),
+                            (int)((hi << 20) | (lo >> 12))) -
+           (1.0 - 0x1p-53);
+  }
+  // Phi^-1 of the grid point of words (hi, lo).  FP64 operations bound the
+  // double-precision stepper (18 clocks a warp on an SM, an integer operation
+  // half a clock, a gathered shared-memory load 4.5), so everything but the
+  // polynomial is integer work: the lower tail p = min(u, 1 - u) as the
+  // 64-bit word p 2^64, its octave by a leading-zero count, the segment from
+  // the next six bits, and t in [-1/2, 1/2) from the remaining (at most 52)
+  // bits put into a mantissa; then a degree-6 polynomial of the segment: 7
+  // FP64 operations, against 45 of norm_quantile_f64, which stays for the
+  // tails beyond the tabulated octaves (p < 2^-11, a tenth of a percent).
+  // Within 2.5e-16 of Phi^-1, max(1, |z|) relative.
+  __device__ __forceinline__ static double quantile(uint32_t hi, uint32_t lo,
+                                                    const F64Tables* tab) {
+    const uint32_t s = (uint32_t)((int)hi >> 31);  // all ones in the upper half
+    const uint32_t ph = hi ^ s;
+    const uint32_t pl = ((lo ^ s) & 0xfffff000u) | 0x800u;
+    double z;
+    if (ph >= (0x80000000u >> kQsOct)) {
+      const int k = __clz((int)ph);  // p in [2^-(k + 1), 2^-k)
+      const uint32_t nh = __funnelshift_l(pl, ph, k), nl = pl << k;
+      const int j = (k << 6) + (int)(nh >> 25) - 128;  // (k - 1) 64 + segment
+      const double t = __hiloint2double((int)(0x3ff00000u | ((nh & 0x1ffffffu) >> 5)),
+                                        (int)__funnelshift_r(nl, nh, 5)) -
+                       1.5;
+      z = tab->qc[kQsDeg][j];
+#pragma unroll
+      for (int i = kQsDeg - 1; i >= 0; --i) z = fma(z, t, tab->qc[i][j]);
+    } else {
+      const double p = grid_point(ph, pl & 0xfffff000u);
+      z = norm_quantile_f64(p, 1.0 - p);
+    }
+    return __hiloint2double(__double2hiint(z) ^ (int)(s & 0x80000000u), __double2loint(z));
+  }
   // U_V, Z_V from words (0, 1); Z_X from words (2, 3)
   __device__ __forceinline__ static void make(uint4 w, double& u, double& omu, double& zV,
-                                              double& zX, const DfTables*) {
-    u = uniform52(w.x, w.y);
-    omu = 1.0 - u;
-    zV = norm_quantile_f64(u, omu);
-    const double uX = uniform52(w.z, w.w);
-    zX = norm_quantile_f64(uX, 1.0 - uX);
+                                              double& zX, const F64Tables* t) {
+    u = grid_point(w.x, w.y);
+    omu = grid_point(~w.x, ~w.y);
+    zV = quantile(w.x, w.y, t);
+    zX = quantile(w.z, w.w, t);
   }
 };
+static_assert(kQsSeg == 64, "the segment index of Draw<double>::quantile");
 template <> struct Draw<float> {
   // U_V from word 0 and Z_X from word 2: the top 23 bits of the words the
   // double-precision grid reads first, so both precisions see one stream
   __device__ __forceinline__ static void make(uint4 w, float& u, float& omu, float& zV,
-                                              float& zX, const DfTables*) {
+                                              float& zX, const NoTables*) {
     u = uniform23(w.x);
     omu = 1.0f - u;
     zV = norm_quantile_f32(u, omu);

@@ -113,23 +113,22 @@ __device__ __forceinline__ Real stored_variance(int scheme, Real v) {
 
 }  // namespace
 
-// Outer states x_n, v_n (n = 0..N) of pricing path p (a thread per path),
+// Outer states x_n (log_price_start), v_n (n = 0..N) of pricing path p (a thread per path),
 // with the forward pass's arithmetic.
 template <typename Real, int SCHEME>
 __global__ void __launch_bounds__(kDualBlock) dual_outer_kernel(DualArgs a) {
   __shared__ GroupConst<Real> gc;
-  constexpr bool kPair = std::is_same<Real, df>::value;
-  __shared__ __align__(16) unsigned char tab_raw[kPair ? sizeof(DfTables) : 16];
-  DfTables* tabs = reinterpret_cast<DfTables*>(tab_raw);
+  extern __shared__ __align__(16) unsigned char tab_raw[];
+  Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
   if (threadIdx.x == 0) make_group_const<Real>(a.group, gc);
-  if constexpr (kPair) load_df_tables(tabs);
+  load_tables<Real>(tabs);
   __syncthreads();
   const uint32_t p = blockIdx.x * kDualBlock + threadIdx.x;
   if (p >= a.n_outer) return;
   const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
   Real* X = (Real*)a.X;
   Real* V = (Real*)a.V;
-  Real x = (Real)0, v = gc.v0;
+  Real x = log_price_start<Real, SCHEME>(gc), v = gc.v0;
   CHK_ST(a.chk, &X[p], x);
   CHK_ST(a.chk, &V[p], v);
   for (uint32_t n = 0; n < a.N; ++n) {
@@ -149,9 +148,8 @@ __global__ void __launch_bounds__(kDualBlock) dual_outer_kernel(DualArgs a) {
 template <typename Real, int SCHEME, int BASIS>
 __global__ void __launch_bounds__(kDualBlock) dual_inner_kernel(DualArgs a) {
   __shared__ GroupConst<Real> gc;
-  constexpr bool kPair = std::is_same<Real, df>::value;
-  __shared__ __align__(16) unsigned char tab_raw[kPair ? sizeof(DfTables) : 16];
-  DfTables* tabs = reinterpret_cast<DfTables*>(tab_raw);
+  extern __shared__ __align__(16) unsigned char tab_raw[];
+  Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
   __shared__ double s_acc[kMaxDualStrikes][kDualBlock];
   __shared__ uint32_t s_ties[kDualBlock];
   __shared__ const Real* s_tab[kMaxDualStrikes];
@@ -170,7 +168,7 @@ __global__ void __launch_bounds__(kDualBlock) dual_inner_kernel(DualArgs a) {
     s_invTh[tid] = (Real)I.inv_theta;
   }
   for (uint32_t k = 0; k < nk; ++k) s_acc[k][tid] = 0.0;
-  if constexpr (kPair) load_df_tables(tabs);
+  load_tables<Real>(tabs);
   __syncthreads();
   const int type = a.type;
   const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
@@ -188,7 +186,7 @@ __global__ void __launch_bounds__(kDualBlock) dual_inner_kernel(DualArgs a) {
       Draw<Real>::make(w, u, omu, zV, zX, tabs);
       if (SCHEME == kSchemeQE) qe_step<Real>(gc, x, v, omu, zV, zX, tabs);
       else ft_step<Real>(gc, x, v, zV, zX);
-      const Real E = Fm<Real>::exp_(x, tabs);
+      const Real E = Fm<Real>::exp_(log_price<Real, SCHEME>(gc, x, v), tabs);
       const Real vs = stored_variance<Real>(SCHEME, v);
       const uint32_t date = m + 1;
       for (uint32_t k = 0; k < nk; ++k) {
@@ -231,10 +229,11 @@ __global__ void __launch_bounds__(kDualBlock) dual_inner_kernel(DualArgs a) {
 // Pathwise maximum of Z_n - pi_n for outer path p and strike k = blockIdx.y.
 template <typename Real, int SCHEME, int BASIS>
 __global__ void __launch_bounds__(kDualBlock) dual_max_kernel(DualArgs a) {
-  constexpr bool kPair = std::is_same<Real, df>::value;
-  __shared__ __align__(16) unsigned char tab_raw[kPair ? sizeof(DfTables) : 16];
-  DfTables* tabs = reinterpret_cast<DfTables*>(tab_raw);
-  if constexpr (kPair) load_df_tables(tabs);
+  extern __shared__ __align__(16) unsigned char tab_raw[];
+  Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
+  __shared__ GroupConst<Real> gc;
+  if (threadIdx.x == 0) make_group_const<Real>(a.group, gc);
+  load_tables<Real>(tabs);
   __syncthreads();
   const uint32_t k = blockIdx.y;
   const uint32_t p = blockIdx.x * kDualBlock + threadIdx.x;
@@ -258,7 +257,10 @@ __global__ void __launch_bounds__(kDualBlock) dual_max_kernel(DualArgs a) {
         !CHK_OK(a.chk, &scr[date], sizeof(ScreenConsts)) ||
         !CHK_OK(a.chk, &Q[n], sizeof(double) * (date < N ? 2 : 1)))
       break;
-    const Real E = Fm<Real>::exp_(CHK_LD(a.chk, &X[(size_t)date * a.n_outer + p]), tabs);
+    const Real E = Fm<Real>::exp_(
+        log_price<Real, SCHEME>(gc, CHK_LD(a.chk, &X[(size_t)date * a.n_outer + p]),
+                                CHK_LD(a.chk, &V[(size_t)date * a.n_outer + p])),
+        tabs);
     const Real S = t[7] * E;
     double Z, L;
     if (date < N) {
@@ -322,10 +324,16 @@ __global__ void dual_sum_kernel(DualArgs a) {
 
 template <typename Real, int SCHEME, int BASIS>
 static cudaError_t launch_dual_t(const DualArgs& a, cudaStream_t s) {
-  dual_outer_kernel<Real, SCHEME><<<(a.n_outer + kDualBlock - 1) / kDualBlock, kDualBlock, 0, s>>>(a);
-  dual_inner_kernel<Real, SCHEME, BASIS><<<a.n_outer * a.N, kDualBlock, 0, s>>>(a);
+  constexpr size_t dyn = tab_bytes<Real>();
+  cudaError_t e = allow_dynamic<dual_outer_kernel<Real, SCHEME>>(dyn);
+  if (e == cudaSuccess) e = allow_dynamic<dual_inner_kernel<Real, SCHEME, BASIS>>(dyn);
+  if (e == cudaSuccess) e = allow_dynamic<dual_max_kernel<Real, SCHEME, BASIS>>(dyn);
+  if (e != cudaSuccess) return e;
+  dual_outer_kernel<Real, SCHEME>
+      <<<(a.n_outer + kDualBlock - 1) / kDualBlock, kDualBlock, dyn, s>>>(a);
+  dual_inner_kernel<Real, SCHEME, BASIS><<<a.n_outer * a.N, kDualBlock, dyn, s>>>(a);
   dual_max_kernel<Real, SCHEME, BASIS>
-      <<<dim3((a.n_outer + kDualBlock - 1) / kDualBlock, a.n_strikes), kDualBlock, 0, s>>>(a);
+      <<<dim3((a.n_outer + kDualBlock - 1) / kDualBlock, a.n_strikes), kDualBlock, dyn, s>>>(a);
   dual_sum_kernel<<<a.n_strikes, kDualBlock, 0, s>>>(a);
   return cudaGetLastError();
 }

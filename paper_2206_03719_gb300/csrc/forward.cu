@@ -48,11 +48,12 @@ forward_kernel(FwdArgs a) {
   if (threadIdx.x < sc.n_groups && threadIdx.x < kMaxGroups &&
       CHK_OK(a.chk, &a.groups[sc.group0 + threadIdx.x], sizeof(FwdGroup)))
     make_group_const<Real>(a.groups[sc.group0 + threadIdx.x], gc[threadIdx.x]);
-  // float pairs: exp and quantile tables in shared memory
+  // the precision's exp and quantile tables in dynamic shared memory
   constexpr bool kPair = std::is_same<Real, df>::value;
-  __shared__ __align__(16) unsigned char tab_raw[kPair ? sizeof(DfTables) : 16];
-  DfTables* tabs = reinterpret_cast<DfTables*>(tab_raw);
-  if constexpr (kPair) load_df_tables(tabs);
+  constexpr bool kDouble = std::is_same<Real, double>::value;
+  extern __shared__ __align__(16) unsigned char tab_raw[];
+  Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
+  load_tables<Real>(tabs);
   __syncthreads();
 
   if (SEG && a.next_job && blockIdx.x == 0 && threadIdx.x == 0)
@@ -157,9 +158,24 @@ forward_kernel(FwdArgs a) {
     // double (and the float Euler scheme): every group's state in registers,
     // the group loop unrolled so the groups' independent chains interleave
     Real x[kMaxGroups], v[kMaxGroups];
+    // plans have unit row scale: no multiplication then (double: it would
+    // take the FP64 pipe)
+    bool scaled = !kDouble;
+    if constexpr (kDouble)
+      for (int g = 0; g < ng; ++g)
+        scaled = scaled || __double_as_longlong(gc[g].out_scale) != __double_as_longlong(1.0);
+    auto row_value = [&](const GroupConst<Real>& c, Real xg, Real vg) {
+      const Real e = Fm<Real>::exp_(log_price<Real, SCHEME>(c, xg, vg), tabs);
+      return narrow<St>(scaled ? c.out_scale * e : e);
+    };
+    auto stored_v = [&](Real vg) {
+      if constexpr (SCHEME != kSchemeFT) return narrow<St>(vg);
+      else if constexpr (kDouble) return narrow<St>(positive_part(vg));
+      else return narrow<St>(vg < (Real)0 ? (Real)0 : vg);
+    };
 #pragma unroll
     for (int g = 0; g < kMaxGroups; ++g) {
-      x[g] = (Real)0;
+      x[g] = g < ng ? log_price_start<Real, SCHEME>(gc[g]) : (Real)0;
       v[g] = g < ng ? gc[g].v0 : (Real)0;
       if (ck_index && g < ng) {
         x[g] = CHK_LD(a.chk, &gc[g].CX[ck_index * gc[g].ld + p]);
@@ -167,10 +183,8 @@ forward_kernel(FwdArgs a) {
       }
       if (first_row && g < ng) {
         const GroupConst<Real>& c = gc[g];
-        CHK_ST(a.chk, &((St*)c.E)[p], narrow<St>(c.out_scale * Fm<Real>::exp_(x[g], tabs)));
-        if (c.V)
-          CHK_ST(a.chk, &((St*)c.V)[p],
-                 narrow<St>((SCHEME == kSchemeFT && v[g] < (Real)0) ? (Real)0 : v[g]));
+        CHK_ST(a.chk, &((St*)c.E)[p], row_value(c, x[g], v[g]));
+        if (c.V) CHK_ST(a.chk, &((St*)c.V)[p], stored_v(v[g]));
       }
     }
     for (uint32_t n = n0; n < n1; ++n) {
@@ -188,10 +202,8 @@ forward_kernel(FwdArgs a) {
           }
           if (store_rows) {
             const size_t off = (size_t)(n + 1 - row0) * c.ld + p;
-            CHK_ST(a.chk, &((St*)c.E)[off], narrow<St>(c.out_scale * Fm<Real>::exp_(x[g], tabs)));
-            if (c.V)
-              CHK_ST(a.chk, &((St*)c.V)[off],
-                     narrow<St>((SCHEME == kSchemeFT && v[g] < (Real)0) ? (Real)0 : v[g]));
+            CHK_ST(a.chk, &((St*)c.E)[off], row_value(c, x[g], v[g]));
+            if (c.V) CHK_ST(a.chk, &((St*)c.V)[off], stored_v(v[g]));
           }
           if (save_at(n + 1)) {
             CHK_ST(a.chk, &c.CX[(size_t)((n + 1) / a.ck_stride) * c.ld + p], x[g]);
@@ -259,14 +271,13 @@ forward_kernel(FwdArgs a) {
 // from counter (path, date, stream, 0xFFFFFFFF).
 
 template <typename Real>
-__device__ __forceinline__ Real common_shock(uint4 w, const DfTables* t);
+__device__ __forceinline__ Real common_shock(uint4 w, const Tab<Real>* t);
 template <>
-__device__ __forceinline__ double common_shock<double>(uint4 w, const DfTables*) {
-  const double u = uniform52(w.z, w.w);
-  return norm_quantile_f64(u, 1.0 - u);
+__device__ __forceinline__ double common_shock<double>(uint4 w, const F64Tables* t) {
+  return Draw<double>::quantile(w.z, w.w, t);
 }
 template <>
-__device__ __forceinline__ float common_shock<float>(uint4 w, const DfTables*) {
+__device__ __forceinline__ float common_shock<float>(uint4 w, const NoTables*) {
   const float u = uniform23(w.z);
   return norm_quantile_f32(u, 1.0f - u);
 }
@@ -275,14 +286,25 @@ __device__ __forceinline__ df common_shock<df>(uint4 w, const DfTables* t) {
   return Draw<df>::quantile(w.z, w.w, t);
 }
 
+// fmax; for the non-negative doubles here by their bits (an FP64 comparison
+// costs the pipe as much as a multiply-add), a NaN giving the other operand
+template <typename Real> __device__ __forceinline__ Real larger(Real a, Real b) {
+  return fmax(a, b);
+}
+template <> __device__ __forceinline__ double larger<double>(double a, double b) {
+  const long long inf = 0x7ff0000000000000ll;
+  const long long ka = __double_as_longlong(a), kb = __double_as_longlong(b);
+  if (ka > inf) return b;
+  return kb > ka && kb <= inf ? b : a;
+}
+
 template <typename Real, int SCHEME, int KA>
 __global__ void __launch_bounds__(kFwdBlock)
 multi_max_kernel(MultiArgs a) {
   __shared__ GroupConst<Real> gc[kMaxAssets];
-  constexpr bool kPair = std::is_same<Real, df>::value;
-  __shared__ __align__(16) unsigned char tab_raw[kPair ? sizeof(DfTables) : 16];
-  DfTables* tabs = reinterpret_cast<DfTables*>(tab_raw);
-  if constexpr (kPair) load_df_tables(tabs);
+  extern __shared__ __align__(16) unsigned char tab_raw[];
+  Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
+  load_tables<Real>(tabs);
   const double dt = a.T / (double)a.N;
   for (uint32_t i = threadIdx.x; i < a.n_assets; i += blockDim.x) {
     const MultiModel& m = a.assets[i];
@@ -306,7 +328,7 @@ multi_max_kernel(MultiArgs a) {
 #pragma unroll
     for (int k = 0; k < KA; ++k) {
       const uint32_t ai = a0 + k < a.n_assets ? a0 + k : a0;
-      x[k] = (Real)0;
+      x[k] = log_price_start<Real, SCHEME>(gc[ai]);
       v[k] = gc[ai].v0;
       if (k == 0 || gc[ai].out_scale > m0) m0 = gc[ai].out_scale;
     }
@@ -330,35 +352,40 @@ multi_max_kernel(MultiArgs a) {
           } else {
             ft_step<Real>(c, x[k], v[k], zV, zX);
           }
-          const Real S = c.out_scale * Fm<Real>::exp_(x[k], tabs);
-          mx = k == 0 ? S : fmax(mx, S);
+          const Real S = c.out_scale * Fm<Real>::exp_(log_price<Real, SCHEME>(c, x[k], v[k]), tabs);
+          mx = k == 0 ? S : larger(mx, S);
         }
       }
       const size_t off = (size_t)(n + 1) * P + p;
-      CHK_ST(a.chk, &M[off], a0 == 0 ? mx : fmax(CHK_LD(a.chk, &M[off]), mx));
+      CHK_ST(a.chk, &M[off], a0 == 0 ? mx : larger(CHK_LD(a.chk, &M[off]), mx));
     }
   }
 }
 
-template <typename Real>
-static void launch_multi_t(const MultiArgs& a, int scheme, cudaStream_t s) {
+template <typename Real, int SCHEME>
+static cudaError_t launch_multi_s(const MultiArgs& a, cudaStream_t s) {
   const unsigned blocks = (a.P + kFwdBlock - 1) / kFwdBlock;
-  if (scheme == kSchemeQE)
-    multi_max_kernel<Real, kSchemeQE, 4><<<blocks, kFwdBlock, 0, s>>>(a);
-  else
-    multi_max_kernel<Real, kSchemeFT, 4><<<blocks, kFwdBlock, 0, s>>>(a);
+  const cudaError_t e = allow_dynamic<multi_max_kernel<Real, SCHEME, 4>>(tab_bytes<Real>());
+  if (e != cudaSuccess) return e;
+  multi_max_kernel<Real, SCHEME, 4><<<blocks, kFwdBlock, tab_bytes<Real>(), s>>>(a);
+  return cudaGetLastError();
+}
+
+template <typename Real>
+static cudaError_t launch_multi_t(const MultiArgs& a, int scheme, cudaStream_t s) {
+  return scheme == kSchemeQE ? launch_multi_s<Real, kSchemeQE>(a, s)
+                             : launch_multi_s<Real, kSchemeFT>(a, s);
 }
 
 cudaError_t launch_multi_max(const MultiArgs& a, int precision, int scheme, cudaStream_t s) {
   if (a.P == 0 || a.N == 0 || a.n_assets == 0) return cudaSuccess;
-  if (precision == kPrecFP64) launch_multi_t<double>(a, scheme, s);
-  else if (precision == kPrecDF) launch_multi_t<df>(a, scheme, s);
-  else launch_multi_t<float>(a, scheme, s);
-  return cudaGetLastError();
+  if (precision == kPrecFP64) return launch_multi_t<double>(a, scheme, s);
+  if (precision == kPrecDF) return launch_multi_t<df>(a, scheme, s);
+  return launch_multi_t<float>(a, scheme, s);
 }
 
-// The exponential of the forward pass (the E rows are S0 exp(x)): exp_f64
-// in double, exp_df on float pairs, __expf in single precision.
+// The exponential of a log price (the E rows are S0 exp(x)): exp_f64 in
+// double, exp_df on float pairs, __expf in single precision.
 template <typename Real>
 __global__ void exp_kernel(const Real* __restrict__ x, Real* __restrict__ y, size_t n) {
   constexpr bool kPair = std::is_same<Real, df>::value;
@@ -369,7 +396,10 @@ __global__ void exp_kernel(const Real* __restrict__ x, Real* __restrict__ y, siz
     __syncthreads();
   }
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (i < n) y[i] = Fm<Real>::exp_(x[i], tabs);
+  if (i >= n) return;
+  if constexpr (std::is_same<Real, double>::value) y[i] = exp_f64(x[i]);
+  else if constexpr (kPair) y[i] = Fm<df>::exp_(x[i], tabs);
+  else y[i] = Fm<float>::exp_(x[i], nullptr);
 }
 
 // The normal quantile of the random inputs on n uniforms (1 - u computed;
@@ -429,39 +459,48 @@ __global__ void draws_kernel(uint2 key, uint32_t stream_id,
   if (i >= n) return;
   const uint4 w = philox4x32_10(make_uint4(path[i], step[i], stream_id, 0u), key);
   Real uV, omu, zV, zX;
-  Draw<Real>::make(w, uV, omu, zV, zX, tabs);
+  const Tab<Real>* t = nullptr;
+  if constexpr (kPair) t = tabs;
+  else if constexpr (std::is_same<Real, double>::value) t = &kF64Tables;  // read once: not staged
+  Draw<Real>::make(w, uV, omu, zV, zX, t);
   out[3 * i] = uV;
   out[3 * i + 1] = zV;
   out[3 * i + 2] = zX;
 }
 
+template <typename Real, int SCHEME, bool SEG, int FMT>
+static cudaError_t launch_forward_k(const FwdArgs& a, cudaStream_t s) {
+  const cudaError_t e =
+      allow_dynamic<forward_kernel<Real, SCHEME, SEG, FMT>>(tab_bytes<Real>());
+  if (e != cudaSuccess) return e;
+  forward_kernel<Real, SCHEME, SEG, FMT><<<a.n_blocks, kFwdBlock, tab_bytes<Real>(), s>>>(a);
+  return cudaGetLastError();
+}
+
 template <typename Real, int FMT>
-static void launch_forward_f(const FwdArgs& a, int scheme, cudaStream_t s) {
+static cudaError_t launch_forward_f(const FwdArgs& a, int scheme, cudaStream_t s) {
   const bool seg = a.n0 != 0 || a.n1 != 0 || a.row0 != 1 || !a.store_rows || a.save_states ||
                    a.next_job;
-  if (scheme == kSchemeQE) {
-    if (seg) forward_kernel<Real, kSchemeQE, true, FMT><<<a.n_blocks, kFwdBlock, 0, s>>>(a);
-    else forward_kernel<Real, kSchemeQE, false, FMT><<<a.n_blocks, kFwdBlock, 0, s>>>(a);
-  } else {
-    if (seg) forward_kernel<Real, kSchemeFT, true, FMT><<<a.n_blocks, kFwdBlock, 0, s>>>(a);
-    else forward_kernel<Real, kSchemeFT, false, FMT><<<a.n_blocks, kFwdBlock, 0, s>>>(a);
-  }
+  if (scheme == kSchemeQE)
+    return seg ? launch_forward_k<Real, kSchemeQE, true, FMT>(a, s)
+               : launch_forward_k<Real, kSchemeQE, false, FMT>(a, s);
+  return seg ? launch_forward_k<Real, kSchemeFT, true, FMT>(a, s)
+             : launch_forward_k<Real, kSchemeFT, false, FMT>(a, s);
 }
 
 template <typename Real>
-static void launch_forward_t(const FwdArgs& a, int scheme, cudaStream_t s) {
-  if (a.store_fmt == kStoreF16) launch_forward_f<Real, kStoreF16>(a, scheme, s);
-  else if (a.store_fmt == kStoreBF16) launch_forward_f<Real, kStoreBF16>(a, scheme, s);
-  else launch_forward_f<Real, kStoreNative>(a, scheme, s);
+static cudaError_t launch_forward_t(const FwdArgs& a, int scheme, cudaStream_t s) {
+  if (a.store_fmt == kStoreF16) return launch_forward_f<Real, kStoreF16>(a, scheme, s);
+  if (a.store_fmt == kStoreBF16) return launch_forward_f<Real, kStoreBF16>(a, scheme, s);
+  return launch_forward_f<Real, kStoreNative>(a, scheme, s);
 }
 
 cudaError_t launch_forward(const FwdArgs& a, int precision, int scheme, cudaStream_t s) {
   if (a.n_blocks == 0) return cudaSuccess;
   if (a.store_fmt < kStoreNative || a.store_fmt > kStoreBF16) return cudaErrorInvalidValue;
-  if (precision == kPrecFP64) launch_forward_t<double>(a, scheme, s);
-  else if (precision == kPrecDF) launch_forward_t<df>(a, scheme, s);
-  else launch_forward_t<float>(a, scheme, s);
-  return cudaGetLastError();
+  if (precision == kPrecFP64) return launch_forward_t<double>(a, scheme, s);
+  if (precision == kPrecDF) return launch_forward_t<df>(a, scheme, s);
+  return launch_forward_t<float>(a, scheme, s);
 }
 
 cudaError_t launch_philox(const uint32_t* ctr, uint32_t k0, uint32_t k1,

@@ -1,0 +1,94 @@
+"""Write forward_f64.h: the tables of the double-precision forward pass,
+computed in 40-digit arithmetic with mpmath.
+
+    python paper_2206_03719_gb300/csrc/gen_forward_f64.py
+
+Quantile: Phi^-1(p) for p in [2^-(OCT+1), 1/2), one degree-6 polynomial per
+segment: octave k = 1..OCT is p in [2^-(k+1), 2^-k), cut in SEG segments of
+equal width.  In a segment t in [-1/2, 1/2) runs linearly over p.  Each
+polynomial interpolates at seven Chebyshev nodes; the coefficients are rounded
+to double one after another from the lowest up.  Stored coefficient-major
+(qc[j][(k - 1) * SEG + segment]).
+
+Exponential: 2^(j / EXPN), j = 0..EXPN-1, and the coefficients of
+2^(f / EXPN) - 1 on |f| <= 1/2 (Taylor to f^3, the f^4 term economised onto
+f^2).
+"""
+import os
+
+import mpmath as mp
+
+mp.mp.dps = 40
+OCT, SEG, DEG = 10, 64, 6
+EXPN = 2048
+
+
+def quantile(p):
+    return -mp.sqrt(2) * mp.erfinv(1 - 2 * p)
+
+
+def segment(k, i):
+    """coefficients of the segment's polynomial in t, and its error"""
+    left = mp.mpf(2) ** -(k + 1) * (1 + mp.mpf(i) / SEG)
+    width = mp.mpf(2) ** -(k + 1) / SEG
+    nodes = [mp.cos(mp.pi * (j + mp.mpf(0.5)) / (DEG + 1)) / 2 for j in range(DEG + 1)]
+    A = mp.matrix(DEG + 1, DEG + 1)
+    b = mp.matrix(DEG + 1, 1)
+    for r, t in enumerate(nodes):
+        for j in range(DEG + 1):
+            A[r, j] = t ** j
+        b[r] = quantile(left + width * (t + mp.mpf(0.5)))
+    c = [float(x) for x in mp.lu_solve(A, b)]
+    worst = mp.mpf(0)
+    for s in (-0.5, -0.37, -0.2, 0.0, 0.11, 0.3, 0.45, 0.5):
+        v = mp.mpf(0)
+        for x in reversed(c):
+            v = v * s + mp.mpf(x)
+        worst = max(worst, abs(v - quantile(left + width * (mp.mpf(s) + mp.mpf(0.5)))))
+    return c, float(worst)
+
+
+def main():
+    rows = [[] for _ in range(DEG + 1)]
+    worst = 0.0
+    for k in range(1, OCT + 1):
+        for i in range(SEG):
+            c, e = segment(k, i)
+            worst = max(worst, e / max(1.0, abs(c[0])))
+            for j in range(DEG + 1):
+                rows[j].append(c[j])
+    print("largest segment error, max(1, |z|) relative: %.3g" % worst)
+    L = mp.log(2) / EXPN
+    a1, a3 = float(L), float(L ** 3 / 6)
+    a2 = float(L ** 2 / 2 + L ** 4 / 96)
+    here = os.path.dirname(os.path.abspath(__file__))
+    with open(os.path.join(here, "forward_f64.h"), "w") as f:
+        f.write("// forward_f64.h -- written by gen_forward_f64.py (40-digit mpmath); do not edit.\n"
+                "#pragma once\n\nnamespace lsmc {\n\n"
+                "constexpr int kQsOct = %d, kQsSeg = %d, kQsDeg = %d;  // octaves, segments, degree\n"
+                "constexpr int kExpN = %d, kExpNLog2 = %d;\n"
+                "constexpr double kExpUnit = %.17e;  // kExpN / ln 2, as a pair\n"
+                "constexpr double kExpUnitLo = %.17e;\n"
+                "constexpr double kExpUnitInv = %.17e;\n"
+                "constexpr double kExpA1 = %.17e;\n"
+                "constexpr double kExpA2 = %.17e;\n"
+                "constexpr double kExpA3 = %.17e;\n\n"
+                "struct F64Tables {\n"
+                "  double qc[kQsDeg + 1][kQsOct * kQsSeg];  // quantile segments\n"
+                "  double exp2[kExpN];                      // 2^(j / kExpN)\n"
+                "};\n\n" % (OCT, SEG, DEG, EXPN, EXPN.bit_length() - 1, float(1 / L), float(1 / L - mp.mpf(float(1 / L))), a1, a1, a2, a3))
+        f.write("static __device__ const F64Tables kF64Tables = {\n    {\n")
+        for r in rows:
+            f.write("        {\n")
+            for i in range(0, len(r), 4):
+                f.write("            " + " ".join("%.17e," % v for v in r[i:i + 4]) + "\n")
+            f.write("        },\n")
+        f.write("    },\n    {\n")
+        e = [float(mp.mpf(2) ** (mp.mpf(j) / EXPN)) for j in range(EXPN)]
+        for i in range(0, EXPN, 4):
+            f.write("        " + " ".join("%.17e," % v for v in e[i:i + 4]) + "\n")
+        f.write("    },\n};\n\n}  // namespace lsmc\n")
+
+
+if __name__ == "__main__":
+    main()

@@ -14,14 +14,56 @@
 
 namespace lsmc {
 
-// Elementary functions per precision; the float-pair ones read their
-// tables from shared memory (t), the others ignore it.
+// Bytes of a precision's tables, and their copy into shared memory (the
+// caller synchronises the block).
+template <typename Real> __host__ __device__ constexpr size_t tab_bytes() {
+  return std::is_same<Real, float>::value ? 0 : sizeof(Tab<Real>);
+}
+template <typename Real> __device__ __forceinline__ void load_tables(Tab<Real>* t) {
+  if constexpr (std::is_same<Real, df>::value) {
+    load_df_tables(t);
+  } else if constexpr (std::is_same<Real, double>::value) {
+    static_assert(sizeof(F64Tables) % sizeof(double2) == 0, "copied by pairs");
+    const double2* src = reinterpret_cast<const double2*>(&kF64Tables);
+    for (int i = threadIdx.x; i < (int)(sizeof(F64Tables) / sizeof(double2)); i += blockDim.x)
+      reinterpret_cast<double2*>(t)[i] = __ldg(&src[i]);
+  }
+}
+// The kernels' dynamic shared memory above 48 KB needs an opt-in.
+template <auto Kernel> static cudaError_t allow_dynamic(size_t bytes) {
+  if (bytes <= 40 * 1024) return cudaSuccess;
+  return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+}
+
+// The unit of a path's log price x: double keeps x in units of
+// ln 2 / kExpN, so that its exponential needs no argument reduction (k is x
+// rounded to an integer, exactly); the constants that x is made of are
+// converted once per group, with the unit as a pair.
+template <typename Real> __device__ __forceinline__ double in_log_units(double c) {
+  return std::is_same<Real, double>::value ? fma(kExpUnit, c, kExpUnitLo * c) : c;
+}
+
+// exp(X ln 2 / kExpN) for a log price X in those units: k = rint(X), f = X - k
+// exact, 2^(f / kExpN) - 1 by a cubic (|f ln 2 / kExpN| <= 1.7e-4; remainder
+// below 5e-18), times 2^(k / kExpN) from the table and the exponent: 7 FP64
+// operations against 10 of exp_f64 (a table of 128 and a two-part reduction).
+// Beyond |x| = 354 CUDA's exp.
+__device__ __forceinline__ double exp_log_price(double X, const F64Tables* tab) {
+  if ((__double2hiint(X) & 0x7fffffff) >= ((1023 + 20) << 20)) return exp(X * kExpUnitInv);
+  const double magic = 6755399441055744.0;  // 1.5 * 2^52: k in the low word
+  const double t = X + magic;
+  const int k = __double2loint(t);
+  const double f = X - (t - magic);
+  const double p = fma(fma(f, kExpA3, kExpA2), f, kExpA1) * f;
+  const double T = tab->exp2[k & (kExpN - 1)];
+  const double y = fma(T, p, T);
+  return __hiloint2double(__double2hiint(y) + ((k >> kExpNLog2) << 20), __double2loint(y));
+}
+
+// Elementary functions per precision (t: the precision's tables).
 template <typename Real> struct Fm;
 template <> struct Fm<double> {
-  __device__ static double div(double a, double b) { return a / b; }
-  __device__ static double sqrt_(double a) { return sqrt(a); }
-  __device__ static double log_(double a, const DfTables*) { return log_f64(a); }
-  __device__ static double exp_(double a, const DfTables*) { return exp_f64(a); }
+  __device__ static double exp_(double a, const F64Tables* t) { return exp_log_price(a, t); }
 };
 template <> struct Fm<float> {
   __device__ static float div(float a, float b) { return __fdividef(a, b); }
@@ -30,8 +72,8 @@ template <> struct Fm<float> {
     asm("sqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(a));
     return r;
   }
-  __device__ static float log_(float a, const DfTables*) { return __logf(a); }
-  __device__ static float exp_(float a, const DfTables*) { return __expf(a); }
+  __device__ static float log_(float a, const NoTables*) { return __logf(a); }
+  __device__ static float exp_(float a, const NoTables*) { return __expf(a); }
 };
 template <> struct Fm<df> {
   __device__ static df div(df a, df b) { return a / b; }
@@ -42,10 +84,15 @@ template <> struct Fm<df> {
 
 template <typename Real>
 struct GroupConst {
-  // QE: m = mA + mB v, s^2 = sA + sB v, x1 = x + c0 + K1 v + K2 v1 + sqrt(K3 (v + v1)) Z
+  // QE: m = mA + mB v, s^2 = sA + sB v (double: half of it), x1 = x + c0 +
+  // K1 v + K2 v1 + sqrt(K3 (v + v1)) Z; in double the state is x - K2 v, K1
+  // holds K1 + K2 (x - K2 v moves by c0 + (K1 + K2) v + sqrt(...) Z: K1 and K2
+  // are large and nearly cancel, and their rounding errors would grow with the
+  // steps), and c0, K1, K2, K3, mudt, hdt,
+  // rho and rhob carry the unit of x (in_log_units)
   Real mA, mB, sA, sB, c0, K1, K2, K3;
   // FT-Euler
-  Real dt, kdt, theta, xi, rho, rhob, mudt;
+  Real dt, kdt, theta, xi, rho, rhob, mudt, hdt;
   Real v0, out_scale;
   void* E;            // rows of the path store (element type: the launch's store format)
   void* V;
@@ -58,30 +105,34 @@ struct GroupConst {
 // with gamma1 = gamma2 = 1/2; the plain Euler coefficients for FT).
 template <typename Real>
 __device__ void make_group_const(const FwdGroup& g, GroupConst<Real>& c) {
+  constexpr bool kDouble = std::is_same<Real, double>::value;
+  auto u = [](double x) { return in_log_units<Real>(x); };
   const double dt = g.dt, k = g.kappa, th = g.theta, xi = g.xi, rho = g.rho;
   const double E = exp(-k * dt);
   const double omE = -expm1(-k * dt);  // 1 - E without cancellation
   c.mA = (Real)(th * omE);
   c.mB = (Real)E;
   if (xi > 0.0) {
-    c.sB = (Real)(xi * xi * E * omE / k);
-    c.sA = (Real)(th * xi * xi * omE * omE / (2.0 * k));
+    const double half = kDouble ? 0.5 : 1.0;
+    c.sB = (Real)(half * (xi * xi * E * omE / k));
+    c.sA = (Real)(half * (th * xi * xi * omE * omE / (2.0 * k)));
     const double K0 = -rho * k * th * dt / xi;
     const double h = 0.5 * dt * (k * rho / xi - 0.5);
-    c.K1 = (Real)(h - rho / xi);
-    c.K2 = (Real)(h + rho / xi);
-    c.c0 = (Real)((g.r - g.q) * dt + K0);
+    c.K1 = (Real)(kDouble ? u(2.0 * h) : u(h - rho / xi));
+    c.K2 = (Real)u(h + rho / xi);
+    c.c0 = (Real)u((g.r - g.q) * dt + K0);
   } else {
     c.sA = c.sB = c.K1 = c.K2 = c.c0 = (Real)0;
   }
-  c.K3 = (Real)(0.5 * dt * (1.0 - rho * rho));
+  c.K3 = (Real)u(u(0.5 * dt * (1.0 - rho * rho)));
   c.dt = (Real)dt;
   c.kdt = (Real)(k * dt);
   c.theta = (Real)th;
   c.xi = (Real)xi;
-  c.rho = (Real)rho;
-  c.rhob = (Real)sqrt(1.0 - rho * rho);
-  c.mudt = (Real)((g.r - g.q) * dt);
+  c.rho = (Real)u(rho);
+  c.rhob = (Real)u(sqrt(1.0 - rho * rho));
+  c.mudt = (Real)u((g.r - g.q) * dt);
+  c.hdt = (Real)u(0.5 * dt);
   c.v0 = (Real)g.v0;
   c.out_scale = (Real)g.out_scale;
   c.E = g.E;
@@ -100,7 +151,7 @@ __device__ void make_group_const(const FwdGroup& g, GroupConst<Real>& c) {
 template <typename Real>
 __device__ __forceinline__ void qe_core(Real mA, Real mB, Real sA, Real sB, Real c0, Real K1,
                                         Real K2, Real K3, Real& x, Real& v, Real omu, Real zV,
-                                        Real zX, const DfTables* t) {
+                                        Real zX, const Tab<Real>* t) {
   using F = Fm<Real>;
   const Real m = fma(mB, v, mA);
   const Real s2 = fma(sB, v, sA);
@@ -123,10 +174,133 @@ __device__ __forceinline__ void qe_core(Real mA, Real mB, Real sA, Real sB, Real
   v = v1;
 }
 
+// ---- double precision --------------------------------------------------------
+// An FP64 instruction holds the pipe of an SM for 18 clocks a warp on GB300;
+// CUDA's square root and division are eight of them each (142 clocks).  The
+// special-function unit's 20-bit seeds take 2 clocks, so square roots and
+// quotients are formed here from a seed y and one third-order correction
+// (the binomial series of (1 - e)^-1/2 and (1 - e)^-1 to e^2, e ~ 2^-20, the
+// remainder below 2^-59), sharing what can be shared.
+
+// max(v, 0) of a double, the sign read as an integer
+__device__ __forceinline__ double positive_part(double v) {
+  return __double2hiint(v) < 0 ? 0.0 : v;
+}
+
+// y ~ 1 / sqrt(a) and the correction: sqrt(a) = g (1 + ep), 1 / sqrt(a) =
+// y (1 + ep), g = a y (0 and 0 for a zero or subnormal a)
+__device__ __forceinline__ void rsqrt_seed(double a, double& y, double& g, double& ep) {
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  if (__double2hiint(a) < 0x00100000) y = 0.0;
+  g = a * y;
+  const double e = fma(-g, y, 1.0);
+  ep = e * fma(e, 0.375, 0.5);
+}
+__device__ __forceinline__ double rcp_f64(double a) {
+  double y;
+  asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  const double e = fma(-a, y, 1.0);
+  return fma(y, fma(e, e, e), y);
+}
+// a double of a known exponent range as a float, within 2^-20 relative
+__device__ __forceinline__ float seed_float(int hi) {
+  return __int_as_float((hi - (896 << 20)) << 3);
+}
+
+// the variance step of the scheme's definition, for means so small or large
+// that the products below could leave the range of double
+static __device__ __noinline__ double qe_variance_plain(double m, double h2, double omu, double zV) {
+  const double s2 = h2 + h2, m2 = m * m;
+  if (s2 <= 1.5 * m2) {
+    const double inv = (m2 + m2) / s2;
+    const double tt = inv - 1.0;
+    const double b2 = tt + sqrt(inv * tt);
+    const double q = sqrt(b2) + zV;
+    return m / (1.0 + b2) * q * q;
+  }
+  const double omp = (m2 + m2) / (s2 + m2);
+  return omu >= omp ? 0.0 : m / omp * log_f64(omp / omu);
+}
+
+// Andersen QE step in double.  With h2 = s^2 / 2 and d = sqrt(m^2 - h2) the
+// quadratic branch's a and b are a = m - d = h2 / (m + d) and a b^2 = d, so
+//   v1 = a (b + Z)^2 = (d + sqrt(a d) Z)^2 / d,
+//   sqrt(a d) = h2 d / sqrt(h2 d (m + d)),
+// two reciprocal square roots (the first giving d and 1 / d) in place of two
+// square roots and two divisions.  Exponential branch: with A = m^2,
+// B = A + 2 h2: 1 - p = 2 A / B and 1 / beta = B / (2 m), and one reciprocal
+// of B U m (U = 1 - U_V) gives both quotients of v1 = B / (2 m) log(2 A / (B U)).
+// About 33 FP64 operations with the quadratic branch against 60 before (the
+// FP64 forward pass of the 131,072 x 252 book 27.5 -> 14.3 ms with the
+// table quantile and exponential).
+template <>
+__device__ __forceinline__ void qe_core<double>(double mA, double mB, double sA, double sB,
+                                                double c0, double K1, double K2, double K3,
+                                                double& x, double& v, double omu, double zV,
+                                                double zX, const F64Tables*) {
+  const double m = fma(mB, v, mA);
+  const double h2 = fma(sB, v, sA);
+  double v1;
+  // 1e-60 < m < 1e60, tested on the exponent
+  if ((unsigned)(__double2hiint(m) - ((1023 - 200) << 20)) < (400u << 20)) {
+    const double D = fma(m, m, -h2);  // psi <= 3/2  <=>  3 D >= h2
+    // decided in float from the high words, clamped to float's range; the
+    // exact comparison (two FP64 operations) only next to the threshold
+    const int hh = __double2hiint(h2);
+    const float fD = seed_float(min(max(__double2hiint(D), 900 << 20), 1140 << 20));
+    const float fh = seed_float(hh), fd = fmaf(3.0f, fD, -fh);
+    bool quad;
+    if ((unsigned)(hh - (900 << 20)) < (240u << 20) && fabsf(fd) > 1e-5f * fh) quad = fd > 0.0f;
+    else quad = 3.0 * D >= h2;
+    if (quad) {
+      double y, g, ep;
+      rsqrt_seed(D, y, g, ep);
+      const double d = fma(g, ep, g), r = fma(y, ep, y);
+      const double n = h2 * d;
+      double y2, g2, ep2;
+      rsqrt_seed(n * (m + d), y2, g2, ep2);
+      const double ny = n * y2;
+      const double sz = fma(ny, ep2, ny) * zV, q = d + sz;
+      v1 = positive_part(fma(q, sz * r, q));  // q^2 / d with sz / d = q / d - 1
+    } else {
+      const double A = m * m, B = fma(2.0, h2, A), bu = B * omu;
+      // 2 A and B / 2 by their exponents
+      const double A2 = __hiloint2double(__double2hiint(A) + (1 << 20), __double2loint(A));
+      if (__double_as_longlong(bu) >= __double_as_longlong(A2)) {
+        v1 = 0.0;
+      } else {
+        const double R = rcp_f64(bu * m);
+        const double Bh = __hiloint2double(__double2hiint(B) - (1 << 20), __double2loint(B));
+        v1 = Bh * (R * bu) * log_f64(A2 * (R * m));
+      }
+    }
+  } else {
+    v1 = qe_variance_plain(m, h2, omu, zV);
+  }
+  double y, g, ep;
+  rsqrt_seed(K3 * (v + v1), y, g, ep);
+  const double gz = g * zX;
+  x = x + (fma(gz, ep, fma(K1, v, c0)) + gz);
+  v = v1;
+}
+
 template <typename Real>
 __device__ __forceinline__ void qe_step(const GroupConst<Real>& c, Real& x, Real& v,
-                                        Real omu, Real zV, Real zX, const DfTables* t) {
+                                        Real omu, Real zV, Real zX, const Tab<Real>* t) {
   qe_core<Real>(c.mA, c.mB, c.sA, c.sB, c.c0, c.K1, c.K2, c.K3, x, v, omu, zV, zX, t);
+}
+
+// The state of a path's log price at date 0, and the log price (in its unit)
+// of a state x with variance v.
+template <typename Real, int SCHEME>
+__device__ __forceinline__ Real log_price_start(const GroupConst<Real>& c) {
+  if constexpr (std::is_same<Real, double>::value && SCHEME == kSchemeQE) return -c.K2 * c.v0;
+  else return (Real)0;
+}
+template <typename Real, int SCHEME>
+__device__ __forceinline__ Real log_price(const GroupConst<Real>& c, Real x, Real v) {
+  if constexpr (std::is_same<Real, double>::value && SCHEME == kSchemeQE) return fma(c.K2, v, x);
+  else return x;
 }
 
 // Full-truncation Euler: v+ = max(v, 0) in drift and diffusion.
@@ -138,6 +312,18 @@ __device__ __forceinline__ void ft_step(const GroupConst<Real>& c, Real& x,
   const Real sq = F::sqrt_(vp * c.dt);
   const Real v1 = v + c.kdt * (c.theta - vp) + c.xi * sq * zV;
   x = x + (c.mudt - (Real)0.5 * vp * c.dt) + sq * (c.rho * zV + c.rhob * zX);
+  v = v1;
+}
+
+template <>
+__device__ __forceinline__ void ft_step<double>(const GroupConst<double>& c, double& x, double& v,
+                                                double zV, double zX) {
+  const double vp = positive_part(v);
+  double y, g, ep;
+  rsqrt_seed(vp * c.dt, y, g, ep);
+  const double sq = fma(g, ep, g);
+  const double v1 = fma(c.xi, sq * zV, fma(c.kdt, c.theta - vp, v));
+  x = x + fma(-c.hdt, vp, c.mudt) + sq * fma(c.rhob, zX, c.rho * zV);
   v = v1;
 }
 

@@ -1,0 +1,120 @@
+"""The double-precision stepper's tables and step (forward_f64.h, Draw<double>
+and qe_core<double>): the quantile segments and the exponential's cubic against
+40-digit values on the CPU; the draws and the paths of the GPU at the models
+where the step changes form."""
+import os
+import re
+
+import numpy as np
+import pytest
+
+import oracle
+
+mp = pytest.importorskip("mpmath")
+HEADER = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))),
+                      "paper_2206_03719_gb300", "csrc", "forward_f64.h")
+OCT, SEG, DEG, EXPN = 10, 64, 6, 2048
+
+
+def _tables():
+    text = open(HEADER).read()
+    const = {k: float(v) for k, v in re.findall(r"constexpr double (\w+) = ([^;]+);", text)}
+    body = text[text.index("kF64Tables = {"):]
+    vals = [float(v) for v in re.findall(r"-?\d\.\d+e[+-]\d+", body)]
+    n = OCT * SEG
+    assert len(vals) == (DEG + 1) * n + EXPN
+    return const, np.array(vals[:(DEG + 1) * n]).reshape(DEG + 1, n), vals[(DEG + 1) * n:]
+
+
+def _quantile(p):
+    return -mp.sqrt(2) * mp.erfinv(1 - 2 * mp.mpf(p))
+
+
+@pytest.mark.parametrize("octave", range(1, OCT + 1))
+def test_quantile_segments_at_their_edges(octave):
+    # the polynomials as rounded, evaluated exactly: within one rounding of
+    # the leading coefficient plus the interpolation error, 1.1e-16 together
+    mp.mp.dps = 40
+    _, qc, _ = _tables()
+    for seg in (0, 1, 31, 62, 63):
+        left = mp.mpf(2) ** -(octave + 1) * (1 + mp.mpf(seg) / SEG)
+        width = mp.mpf(2) ** -(octave + 1) / SEG
+        c = qc[:, (octave - 1) * SEG + seg]
+        for t in (-0.5, 0.0, 0.5):
+            v = mp.mpf(0)
+            for x in c[::-1]:
+                v = v * t + mp.mpf(float(x))
+            z = _quantile(left + width * (mp.mpf(t) + mp.mpf(0.5)))
+            assert abs(v - z) <= mp.mpf(1.1e-16) * max(1, abs(z))
+
+
+def test_exponential_cubic_and_table():
+    mp.mp.dps = 40
+    const, _, e2 = _tables()
+    for j in (0, 1, 1023, 2047):
+        assert e2[j] == float(mp.mpf(2) ** (mp.mpf(j) / EXPN))
+    for f in (-0.5, -0.3, 0.1, 0.5):
+        p = ((const["kExpA3"] * mp.mpf(f) + mp.mpf(const["kExpA2"])) * f +
+             mp.mpf(const["kExpA1"])) * f
+        assert abs(p - (mp.mpf(2) ** (mp.mpf(f) / EXPN) - 1)) < 2e-17
+    unit = mp.mpf(const["kExpUnit"]) + mp.mpf(const["kExpUnitLo"])
+    assert abs(unit * mp.log(2) / EXPN - 1) < 1e-30
+
+
+@pytest.mark.gpu
+def test_draws_within_one_rounding_of_the_segments():
+    from gpu_common import torch_cuda
+    from paper_2206_03719_gb300 import build
+    from paper_2206_03719_gb300 import lsmc as L
+    torch = torch_cuda()
+    build.build()
+    mp.mp.dps = 30
+    n = 3000
+    path = torch.arange(n, dtype=torch.int32, device="cuda")
+    step = torch.full_like(path, 3)
+    out = torch.empty((n, 3), dtype=torch.float64, device="cuda")
+    L.lsmc_draws(99, 1, path.data_ptr(), step.data_ptr(), n, L.LSMC_FP64, out.data_ptr())
+    got = out.cpu().numpy()
+    worst = 0.0
+    for u, zv, _ in got:
+        z = _quantile(mp.mpf(float(u)))
+        # table 1.1e-16, the last multiply-add half a unit in the last place
+        # (1.2e-16), the inner ones a hundredth of it; the tails use
+        # norm_quantile_f64 (6e-16)
+        tail = min(u, 1.0 - u) < 2.0 ** -(OCT + 1)
+        err = float(abs(mp.mpf(float(zv)) - z) / max(1, abs(z)))
+        assert err <= (6e-16 if tail else 2.5e-16), (u, zv, err)
+        worst = max(worst, err)
+    print("draws: worst %.3g" % worst)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kw", [
+    dict(xi=1e-9),                                 # psi -> 0: a is far below m
+    dict(xi=2.5, kappa=0.3, theta=0.02),           # nearly always the exponential branch
+    dict(v0=0.0),                                  # zero start
+    dict(v0=1e-70, theta=1e-70, xi=1e-36),         # outside the range of the products
+    dict(rho=1.0), dict(rho=-1.0),                 # K3 = 0
+], ids=lambda k: ",".join("%s=%g" % i for i in k.items()))
+def test_paths_where_the_step_changes_form_match_oracle(kw):
+    from gpu_common import torch_cuda
+    from paper_2206_03719_gb300 import build
+    from paper_2206_03719_gb300 import lsmc as L
+    torch = torch_cuda()
+    build.build()
+    model = dict(S0=100.0, r=0.02, q=0.0, v0=0.04, kappa=1.5, theta=0.04, xi=0.3, rho=-0.7)
+    model.update(kw)
+    P, N = 500, 30
+    S = torch.empty((N + 1, P), dtype=torch.float64, device="cuda")
+    V = torch.empty_like(S)
+    L.lsmc_paths(L.lsmc_heston(**model), 0.5, L.LSMC_SCHEME_QE, L.LSMC_FP64, P, N, 5, 2,
+                 S.data_ptr(), V.data_ptr())
+    So, Vo = oracle.paths(oracle.heston(**model), 0.5, oracle.QE, P, N, 5, 2)
+    # the stage tests' tolerances; log prices carry 1/xi of the variance's
+    # rounding (K2 = rho / xi) at the smallest xi
+    rtol_s = 1e-12 + 2e-16 * 100 * model["v0"] / model["xi"]
+    assert np.allclose(S.cpu().numpy(), So, rtol=rtol_s, atol=0)
+    # where the variance nearly vanishes (v1 = log(omp / U) / beta at omp ~ U) the
+    # oracle's own rounding is amplified by the step: 1e-13 absolute
+    assert np.allclose(V.cpu().numpy(), Vo, rtol=1e-11,
+                       atol=1e-13 if model["theta"] > 1e-10 else 1e-84)
