@@ -39,6 +39,7 @@
 #include "device_common.cuh"
 #include "dfloat.cuh"
 #include "exercise.cuh"
+#include "fixed_moments.cuh"
 #include "kernels.h"
 #include "plan.h"
 #include "store16.cuh"
@@ -56,7 +57,6 @@ __host__ __device__ constexpr int mono(int a, int b) {
 // right-hand sides R.  Returns false (no exercise on this date) when fewer
 // in-the-money paths than basis functions were seen, or when a Cholesky pivot
 // is not above 1e-13 times the largest diagonal entry.
-template <bool kNoDivide>
 __device__ bool solve_normal_equations(int B, const double* M, const double* R,
                                        double beta[6]) {
   const int pa[6] = {0, 1, 2, 0, 1, 0};
@@ -67,25 +67,12 @@ __device__ bool solve_normal_equations(int B, const double* M, const double* R,
   for (int i = 0; i < B; ++i)
     for (int j = 0; j < B; ++j) A[i][j] = M[mono(pa[i] + pa[j], pb[i] + pb[j])];
   for (int i = 0; i < B; ++i) maxdiag = fmax(maxdiag, A[i][i]);
-  // kNoDivide (the double-precision kernel): the solve is the critical path
-  // of its regression's chain of dates and runs on one thread while the other
-  // CTAs keep the FP64 pipe busy, where each dependent operation waits some
-  // 200 cycles; one reciprocal square root per pivot gives both
-  // L_jj = d / sqrt(d) and 1 / L_jj, and the substitutions multiply by the
-  // reciprocals, so no division remains on the chain (within a few ulps of
-  // the divided form): the last CTA's reduction and solve 33 -> 21 us, the
-  // FP64 backward 1.4% faster.  The float-pair kernel, whose FP64 pipe is
-  // idle, keeps the square root and the divisions (it measured 1.3% slower
-  // with the reciprocals).
-  double rinv[6];
   for (int j = 0; j < B; ++j) {
     double d = A[j][j];
     for (int k = 0; k < j; ++k) d -= L[j][k] * L[j][k];
     if (!(d > 1e-13 * maxdiag)) return false;
-    const double rj = kNoDivide ? rsqrt(d) : 0.0;
-    L[j][j] = kNoDivide ? d * rj : sqrt(d);
-    const double inv = kNoDivide ? rj : 1.0 / L[j][j];
-    rinv[j] = inv;
+    L[j][j] = sqrt(d);
+    const double inv = 1.0 / L[j][j];
     for (int i = j + 1; i < B; ++i) {
       double s = A[i][j];
       for (int k = 0; k < j; ++k) s -= L[i][k] * L[j][k];
@@ -96,15 +83,83 @@ __device__ bool solve_normal_equations(int B, const double* M, const double* R,
   for (int i = 0; i < B; ++i) {
     double s = R[i];
     for (int k = 0; k < i; ++k) s -= L[i][k] * z[k];
-    z[i] = kNoDivide ? s * rinv[i] : s / L[i][i];
+    z[i] = s / L[i][i];
   }
   for (int i = B - 1; i >= 0; --i) {
     double s = z[i];
     for (int k = i + 1; k < B; ++k) s -= L[k][i] * beta[k];
-    beta[i] = kNoDivide ? s * rinv[i] : s / L[i][i];
+    beta[i] = s / L[i][i];
   }
   for (int i = B; i < 6; ++i) beta[i] = 0.0;
   return true;
+}
+
+// The same by a warp (double and float pairs): the solve is on the critical
+// path of its regression's chain of dates, and on one thread its 200 or so
+// FP64 instructions, each holding a quarter of the SM's pipe for 72 clocks,
+// take 7 us or more.  Lane (i, j), j < B, j <= i <= B, holds entry (i, j) of
+// the factor, row B being the right-hand side, so the elimination does the
+// forward substitution as well; one reciprocal square root a pivot, products
+// instead of divisions: about 65 FP64 instructions.  Coefficient i ends in
+// lane i.  (Single precision keeps the serial form: its coefficients are
+// rounded to float, and its results stay the same bits.)
+template <int B>
+__device__ bool solve_normal_equations_warp(const double* M, const double* R, int lane,
+                                            double& beta) {
+  if (M[0] < (double)B) return false;
+  // column j starts at lane j (B + 1) - j (j - 1) / 2
+  auto at = [](int i, int j) { return j * (B + 1) - j * (j - 1) / 2 + i - j; };
+  int j = 0;
+#pragma unroll
+  for (int c = 1; c < B; ++c) j = lane >= at(c, c) ? c : j;
+  const int i = lane - at(j, j) + j;
+  const bool own = lane < at(B - 1, B - 1) + 2;
+  // powers of x and w of basis function k: {0, 1, 2, 0, 1, 0}, {0, 0, 0, 1, 1, 2}
+  auto px = [](int k) { return (0x010210 >> (4 * k)) & 15; };
+  auto pw = [](int k) { return (0x211000 >> (4 * k)) & 15; };
+  double v = 0.0;
+  if (own) v = i == B ? R[j] : M[mono(px(i) + px(j), pw(i) + pw(j))];
+  long long md = 0;  // the largest diagonal entry: non-negative, compared as integers
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    const long long t = __double_as_longlong(M[mono(2 * px(k), 2 * pw(k))]);
+    md = t > md ? t : md;
+  }
+  const double floor_d = 1e-13 * __longlong_as_double(md);
+  double rinv = 0.0;  // lane k < B: 1 / L_kk
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < B; ++k) {
+    const double d = __shfl_sync(0xffffffffu, v, at(k, k));
+    ok = ok && d > floor_d;
+    double y, g, ep;
+    rsqrt_seed(d, y, g, ep);
+    const double rk = fma(y, ep, y);
+    if (lane == k) rinv = rk;
+    if (j == k) v = i == k ? d * rk : v * rk;
+    const double li = __shfl_sync(0xffffffffu, v, at(i, k) & 31);
+    const double lj = __shfl_sync(0xffffffffu, v, at(j, k) & 31);
+    if (own && j > k) v = fma(-li, lj, v);
+  }
+  if (!ok) return false;  // uniform
+  double s = __shfl_sync(0xffffffffu, v, lane < B ? at(B, lane) : 0);
+  beta = 0.0;
+#pragma unroll
+  for (int k = B - 1; k >= 0; --k) {
+    if (lane == k) beta = s * rinv;
+    const double bk = __shfl_sync(0xffffffffu, beta, k);
+    const double l = __shfl_sync(0xffffffffu, v, lane < k ? at(k, lane) : 0);
+    if (lane < k) s = fma(-l, bk, s);
+  }
+  return true;
+}
+
+constexpr uint32_t kCumTab = 512;  // entries of the tile prefix sums in shared memory
+
+// The in-the-money threshold of a date on the row value: itm_threshold for
+// double, K / s for float pairs.
+template <typename Real> __device__ double row_threshold(int type, double s, double K) {
+  return std::is_same<Real, double>::value ? itm_threshold(type, s, K) : K / s;
 }
 
 struct JobInfo {
@@ -115,6 +170,18 @@ struct JobInfo {
 
 }  // namespace
 
+// Where the time goes (131,072 x 252 x 55 regressions, untuned shape 5 x 4): with
+// double sums the FP64 pipe was 72 to 78% busy and the double kernel took
+// 55.3 ms; with the fixed-point sums 35.9 ms, issue-bound like the float-pair
+// one (about 350 instructions per path and date, 2 a clock).  What a job
+// costs beside its paths (taking and decoding it, the wait, the constants, the
+// reduction, the arrival) was 11 us of its CTA; the serial parts of it --
+// dependent table loads, two thresholds with a division and a bounded walk
+// each, atomics one after the other, the solve on one thread -- now run over
+// the lanes, overlap or sit beside the solve: 35.9 -> 32.0 ms (float pairs 32.3
+// -> 31.3, single precision 83.5 -> 80.1 at 1,048,576 paths; jobs of one
+// sub-tile of 128 paths 152 -> 108).
+//
 // Threads per CTA of the backward pass and resident CTAs per SM: 64 x 8 for
 // double (shorter barriers around the FP64 pipe's work: the FP64 backward of
 // the paper-size book 62.3 ms with 256 x 2, 59.4 with 128 x 4, 58.1 with
@@ -169,21 +236,12 @@ __device__ __forceinline__ float2 pair_add(float2 x, float2 y) {
 
 namespace {
 
-// Per-thread moment sums across the sub-tiles of a job.  Double precision
-// adds into one double per sum.  Single precision sums at most 4 PPT paths in
+// Per-thread moment sums across the sub-tiles of a job (double precision:
+// FixedSums, fixed_moments.cuh).  Single precision sums at most 4 PPT paths in
 // float, then folds that partial into an unevaluated pair (hi + lo) with
 // Knuth's two-sum, so a job of many sub-tiles keeps about 44 bits beyond the
 // partials' own rounding.
 template <typename Real, int NA> struct Acc;
-template <int NA> struct Acc<double, NA> {
-  double s[NA];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int i = 0; i < NA; ++i) s[i] = 0.0;
-  }
-  __device__ __forceinline__ double* target() { return s; }
-  __device__ __forceinline__ void fold() {}
-};
 template <int NA> struct Acc<df, NA> {
   df s[NA];  // float-pair accumulation needs no folding
   __device__ __forceinline__ void zero() {
@@ -217,40 +275,10 @@ template <int NA> struct Acc<float, NA> {
   }
 };
 
-// Reduce-scatter of C per-lane doubles over the warp by recursive halving
-// over the lane bits O, O / 2, ..., 1: at each level lane l and its partner
-// l ^ O split the sums they still hold, the lane with the bit clear keeps the
-// lower half and its partner the upper half (padded with zeros), and each
-// adds the partner's copy of the half it keeps.  After the last level a lane
-// holds one complete sum over the 32 lanes, summed in a fixed order; `idx` is
-// its index (base + position), or -1 for a lane left with padding only.
-template <int C, int O>
-__device__ __forceinline__ void halving_sum(const double (&v)[C], int lane, int base, int real,
-                                            double& out, int& idx) {
-  constexpr int H = (C + 1) / 2;
-  const bool upper = (lane & O) != 0;
-  double nxt[H];
-#pragma unroll
-  for (int i = 0; i < H; ++i) {
-    const double lo = v[i];
-    const double hi = (H + i < C) ? v[(H + i < C) ? H + i : i] : 0.0;
-    const double got = __shfl_xor_sync(0xffffffffu, upper ? lo : hi, O);
-    nxt[i] = (upper ? hi : lo) + got;
-  }
-  const int nbase = upper ? base + H : base;
-  const int nreal = upper ? (real > H ? real - H : 0) : (real < H ? real : H);
-  if constexpr (O == 1) {
-    static_assert(H == 1, "at most 32 sums");
-    out = nxt[0];
-    idx = nreal >= 1 ? nbase : -1;
-  } else {
-    halving_sum<H, O / 2>(nxt, lane, nbase, nreal, out, idx);
-  }
-}
-
 }  // namespace
 
-// Adds one in-the-money path to the per-thread moment sums: the 15
+// Adds one in-the-money path to the per-thread moment sums (float pairs and
+// single precision): the 15
 // monomials x^a w^b (a + b <= 4) of the centred basis variables
 // x = S/K - 1, w = v/theta - 1 and the six products with the cash flow y.
 // Every monomial of degree 3 or 4 is the product of two basis functions
@@ -476,9 +504,10 @@ backward_kernel(BwdArgs a) {
   constexpr int NW = kBT / 32;
 
   __shared__ JobInfo s_job;
-  __shared__ double s_beta[6];
+  __shared__ uint32_t s_cum[kCumTab];
   __shared__ int s_beta_ok;
   __shared__ int s_last;
+  __shared__ int s_go;                // 0: the wait for the previous date failed
   __shared__ double s_red[NW][kNSum];
   __shared__ float2 s_redf[NW][NA];   // single precision: per-warp pair sums
   __shared__ double s_chunk[NW][kNSum];
@@ -487,7 +516,12 @@ backward_kernel(BwdArgs a) {
   __shared__ long long s_thr[2];      // double: in-the-money thresholds of dates n + 1, n
   __shared__ int s_thrf[2];           // the same for float row values (16-bit store)
   __shared__ df s_thrdf[2];           // float pairs: the thresholds K / s of dates n + 1, n
+  __shared__ double s_thrd[2];        // the thresholds as doubles
   __shared__ ScreenConsts s_q;        // the exercise test of date n + 1 in float
+  constexpr bool kFixed = std::is_same<Real, double>::value;
+  constexpr bool kSerialSolve = std::is_same<Real, float>::value;
+  __shared__ FixScale s_fix;          // double: the moment sums' fixed-point scales
+  __shared__ int s_range[3];
   // per-warp compaction of in-the-money paths (dynamic shared memory, one
   // BwdWarpBufs per warp): the heavy arithmetic runs on dense lists instead
   // of on lanes that are mostly out of the money
@@ -506,32 +540,46 @@ backward_kernel(BwdArgs a) {
   // threshold on the stored value), so the compaction buffers hold the
   // stored value and S = s e is formed on the dense lists, where no lane idles
   constexpr bool kProdLate = kCompact;
-  // Job taking and decoding by thread 0, when the CTA has arrived with its
-  // previous job: a job is taken only once the CTA can start it.
-  auto decode = [&]() {
+  // Job decoding by thread 0.  A job number is taken when the CTA has arrived
+  // with its previous job (only once the CTA can start it).  Job numbers only
+  // grow, so the round is found from the last one's; the instance by a binary
+  // search over every s_step-th entry of cum_tiles in shared memory (dependent
+  // global loads here were on the path of every job).  An error recorded by
+  // another CTA is seen in the wait for the previous date.
+  const uint32_t cum_step = (a.n_inst + kCumTab - 1) / kCumTab;
+  uint32_t round = 0;                          // thread 0: the last job's round,
+  unsigned long long round_lo = 0, round_hi = 0;  // its first job and the next round's
+  auto decode = [&](unsigned long long job) {
     JobInfo ji;
     ji.abort = 0;
     ji.round = ji.inst = ji.tile = 0;
-    ji.job = ld_volatile(&a.ctl->error) != 0 ? a.total_jobs
-                                             : atomicAdd(&a.ctl->next_job, 1ull);
+    ji.job = job;
     if (ji.job >= a.total_jobs) {
       ji.abort = 1;
     } else {
-      // round: last r with round_off[r] <= job
-      uint32_t lo = 0, hi = a.n_rounds;
-      while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) / 2;
-        if (CHK_LD(a.chk, &a.round_off[mid]) <= ji.job) lo = mid; else hi = mid;
+      while (job >= round_hi) {
+        ++round;
+        round_lo = round_hi;
+        round_hi = CHK_LD(a.chk, &a.round_off[round + 1]);
       }
-      const uint32_t local = (uint32_t)(ji.job - CHK_LD(a.chk, &a.round_off[lo]));
-      uint32_t klo = 0, khi = CHK_LD(a.chk, &a.active[lo]);
+      const uint32_t local = (uint32_t)(job - round_lo);
+      const uint32_t act = CHK_LD(a.chk, &a.active[round]);
+      uint32_t klo = 0, khi = (act + cum_step - 1) / cum_step;
       while (khi - klo > 1) {
         const uint32_t mid = (klo + khi) / 2;
-        if (CHK_LD(a.chk, &a.cum_tiles[mid]) <= local) klo = mid; else khi = mid;
+        if (s_cum[mid] <= local) klo = mid; else khi = mid;
       }
-      ji.round = lo;
+      uint32_t base = s_cum[klo];
+      klo *= cum_step;
+      khi = min(klo + cum_step, act);
+      while (khi - klo > 1) {
+        const uint32_t mid = (klo + khi) / 2;
+        const uint32_t c = CHK_LD(a.chk, &a.cum_tiles[mid]);
+        if (c <= local) { klo = mid; base = c; } else { khi = mid; }
+      }
+      ji.round = round;
       ji.inst = klo;
-      ji.tile = local - CHK_LD(a.chk, &a.cum_tiles[klo]);
+      ji.tile = local - base;
       // the job's instance and state must lie in the tables
       if (!CHK_OK(a.chk, &a.inst[klo], sizeof(BwdInstance)) ||
           !CHK_OK(a.chk, &a.state[klo], sizeof(BwdState)))
@@ -541,7 +589,22 @@ backward_kernel(BwdArgs a) {
   };
   // the control word (job counter, error word) must lie in the plan
   if (!CHK_OK(a.chk, a.ctl, sizeof(Control))) return;
-  if (tid == 0) decode();
+  for (uint32_t i = tid; i * cum_step < a.n_inst; i += kBT)
+    s_cum[i] = CHK_LD(a.chk, &a.cum_tiles[i * cum_step]);
+  __syncthreads();
+  if (tid == 0) {
+    // the round of the first job: the last one with round_off <= job
+    const unsigned long long job = atomicAdd(&a.ctl->next_job, 1ull);
+    uint32_t lo = 0, hi = a.n_rounds;
+    while (hi - lo > 1) {
+      const uint32_t mid = (lo + hi) / 2;
+      if (CHK_LD(a.chk, &a.round_off[mid]) <= job) lo = mid; else hi = mid;
+    }
+    round = lo;
+    round_lo = CHK_LD(a.chk, &a.round_off[lo]);
+    round_hi = CHK_LD(a.chk, &a.round_off[lo + 1]);
+    decode(job);
+  }
   __syncthreads();
 
   for (;;) {
@@ -567,88 +630,106 @@ backward_kernel(BwdArgs a) {
     const uint32_t tile_base = ji.tile * (sub * TILE0);
 
     // ---- warp 0: wait for the exercise rule of date n + 1, then convert the
-    // per-job constants to the working precision once ------------------------
+    // per-job constants to the working precision once, a constant per lane ----
     if (warp == 0) {
-      if (tid == 0) {
-        int ok = 1;
-        if (!first) {
-          const unsigned long long t0 = global_timer_ns();
-          unsigned spins = 0, ns = 32;
-          while (ld_acquire_gpu(&st->ready) < r) {
-            // back off (32 ns doubling to 512 ns); the error word and the
-            // clock are read every 32nd time
-            __nanosleep(ns);
-            ns = ns < 512 ? 2 * ns : 512;
-            if ((++spins & 31) == 0) {
-              if (ld_volatile(&a.ctl->error) != 0) { ok = 0; break; }
-              if (spins > (1u << 26) || global_timer_ns() - t0 > a.timeout_ns) {
-                atomicCAS(&a.ctl->error, 0u, (uint32_t)kDevErrTimeout);
-                a.ctl->error_info = ji.inst;
-                ok = 0;
-                break;
-              }
+      // what does not depend on the previous round is loaded before the wait
+      double v = 0.0;
+      switch (lane) {
+        case 6: v = CHK_LD(a.chk, &stab[n + 1]); break;
+        case 7: case 13: v = CHK_LD(a.chk, &dtab[n + 1]); break;
+        case 8: v = CHK_LD(a.chk, &stab[N]); break;
+        case 9: v = CHK_LD(a.chk, &stab[n]); break;
+        case 10: v = I.K; break;
+        case 11: v = I.invK; break;
+        case 12: v = I.inv_theta; break;
+        case 14: case 15: v = CHK_LD(a.chk, &dtab[N]); break;
+        case 17:  // later rounds: formed beside the previous date's solve
+          if (kProdLate && first && !final_job)
+            v = row_threshold<Real>(type, CHK_LD(a.chk, &stab[n]), I.K);
+          break;
+        default: break;
+      }
+      // discount factors as unevaluated pairs (hi + lo): a cash flow is
+      // h * hi + h * lo, one rounding, with no bias shared by the paths
+      // that exercise on the same date
+      if (lane == 13 || lane == 15) v = v - (double)(Real)v;
+      int ok = 1;
+      if (tid == 0 && !first) {
+        const unsigned long long t0 = global_timer_ns();
+        unsigned spins = 0, ns = 32;
+        while (ld_acquire_gpu(&st->ready) < r) {
+          // back off (32 ns doubling to 512 ns); the error word and the
+          // clock are read every 32nd time
+          __nanosleep(ns);
+          ns = ns < 512 ? 2 * ns : 512;
+          if ((++spins & 31) == 0) {
+            if (ld_volatile(&a.ctl->error) != 0) { ok = 0; break; }
+            if (spins > (1u << 26) || global_timer_ns() - t0 > a.timeout_ns) {
+              atomicCAS(&a.ctl->error, 0u, (uint32_t)kDevErrTimeout);
+              a.ctl->error_info = ji.inst;
+              ok = 0;
+              break;
             }
           }
-          if (ok) {
-            __threadfence();
-            s_beta_ok = (int)__ldcg(&st->beta_ok);
-            for (int i = 0; i < 6; ++i) s_beta[i] = __ldcg(&st->beta[i]);
-          }
         }
-        s_last = ok ? 0 : -1;
       }
-      __syncwarp();
-      if (lane < 16) {
-        double v;
-        switch (lane) {
-          case 6: v = CHK_LD(a.chk, &stab[n + 1]); break;
-          case 7: v = CHK_LD(a.chk, &dtab[n + 1]); break;
-          case 8: v = CHK_LD(a.chk, &stab[N]); break;
-          case 9: v = CHK_LD(a.chk, &stab[n]); break;
-          case 10: v = I.K; break;
-          case 11: v = I.invK; break;
-          case 12: v = I.inv_theta; break;
-          // discount factors as unevaluated pairs (hi + lo): a cash flow is
-          // h * hi + h * lo, one rounding, with no bias shared by the paths
-          // that exercise on the same date
-          case 13: {
-            const double d = CHK_LD(a.chk, &dtab[n + 1]);
-            v = d - (double)(Real)d;
-            break;
-          }
-          case 14: v = CHK_LD(a.chk, &dtab[N]); break;
-          case 15: {
-            const double d = CHK_LD(a.chk, &dtab[N]);
-            v = d - (double)(Real)d;
-            break;
-          }
-          default: v = first ? 0.0 : s_beta[lane]; break;
-        }
-        s_c[lane] = (Real)v;
-      } else if (kProdLate && lane < 18) {
-        const double sv = CHK_LD(a.chk, lane == 16 ? &stab[n + 1] : &stab[n]);
+      // the flag was acquired by lane 0; the warp barrier orders the lanes'
+      // loads of what was published with it
+      ok = __shfl_sync(0xffffffffu, ok, 0);
+      if (!first && ok) {
+        if (lane < 6) v = __ldcg(&st->beta[lane]);
+        if (kProdLate && (lane == 16 || lane == 17)) v = __ldcg(&st->thr[lane - 16]);
+        if (lane == 18) s_beta_ok = (int)__ldcg(&st->beta_ok);
+        if (kFixed && lane >= 19 && lane < 22) s_range[lane - 19] = __ldcg(&st->range[lane - 19]);
+      } else if (kFixed && lane == 19) {
+        // the first date: |x| < 1 for a put, w within 8, y within the strike
+        s_range[0] = type == kPut ? 0 : 1;
+        s_range[1] = 3;
+        s_range[2] = min(max(ilogb(I.K) + 1, kFixRangeMin), kFixRangeMax);
+      }
+      if (lane == 0) s_go = ok;
+      const Real vr = (Real)v;
+      if (lane < 16) s_c[lane] = vr;
+      if (kProdLate && (lane == 16 || lane == 17)) {
+        // double: S = RN(s e) is in the money exactly where e passes the
+        // date's threshold T (integer comparison of the bits; a float e of a
+        // 16-bit store against T rounded up or down).  Float pairs: S = s e <
+        // K where e < K / s (put), > for a call; the two tests can differ only
+        // where s e lies within the pairs' rounding (about 1e-14) of K.
         if constexpr (std::is_same<Real, double>::value) {
-          const double T = itm_threshold(type, sv, I.K);
-          s_thr[lane - 16] = __double_as_longlong(T);
-          // float e: e < T iff e < (T rounded up to a float); e > T iff e > (T rounded down)
+          s_thr[lane - 16] = __double_as_longlong(v);
           if constexpr (kNarrow64)
             s_thrf[lane - 16] =
-                __float_as_int(type == kPut ? __double2float_ru(T) : __double2float_rd(T));
-        } else {
-          // float pairs: S = s e < K where e < K / s (put), > for a call; the
-          // two tests can differ only where s e lies within the pairs'
-          // rounding (about 1e-14 relative) of K
-          s_thrdf[lane - 16] = df(I.K / sv);
+                __float_as_int(type == kPut ? __double2float_ru(v) : __double2float_rd(v));
+        } else if constexpr (std::is_same<Real, df>::value) {
+          s_thrdf[lane - 16] = vr;
         }
+        s_thrd[lane - 16] = v;
       }
-      __syncwarp();
-      // the compaction buffers hold the row value e (double) or S itself
-      if (kCompact && lane == 0)
-        make_screen<BASIS, Real>(s_q, s_c, kProdLate ? s_c[6] : (Real)1, s_c[10], s_c[11],
-                                 s_c[12], s_c[7]);
+      if constexpr (kCompact) {
+        // the float screen of the exercise test (the compaction buffers hold
+        // the row value e): coefficients, S multiplier, strike, ...
+        const float f = (float)(double)vr;
+        const float ab = lane < 6 ? fabsf(f) : 0.0f;
+        float B = 0.0f;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) B += __shfl_sync(0xffffffffu, ab, i);
+        if (lane < 6) s_q.b[lane] = f;
+        else if (lane == 6) s_q.s = f;
+        else if (lane == 7) s_q.d = f;
+        else if (lane == 10) s_q.K = f;
+        else if (lane == 11) s_q.invK = f;
+        else if (lane == 12) s_q.invTh = f;
+        else if (lane == 13) s_q.B = B;
+      }
+      if constexpr (kFixed) {
+        __syncwarp();
+        if (lane == 19)
+          s_fix = FixScale{kFixBits - s_range[0], kFixBits - s_range[1], kFixBits - s_range[2]};
+      }
     }
     __syncthreads();
-    if (s_last < 0) return;
+    if (!s_go) return;
     const int bok = first ? 0 : s_beta_ok;
     Real b[6];
 #pragma unroll
@@ -671,7 +752,7 @@ backward_kernel(BwdArgs a) {
     const St* V0 = (BASIS == kBasisSV2 && !final_job)
                          ? V + ((ptrdiff_t)n - r0) * (ptrdiff_t)ld : nullptr;
 
-    Acc<Real, NA> acc;
+    typename std::conditional<kFixed, FixedSums<BASIS>, Acc<Real, NA>>::type acc;
     acc.zero();
     uint32_t n_itm = 0;  // in-the-money paths of this thread (monomial 1)
     double euro = 0.0, sy = 0.0, sy2 = 0.0;
@@ -809,7 +890,7 @@ backward_kernel(BwdArgs a) {
           const uint32_t code = wb.xo[j];
           const int pre = (int)(code >> 30);
           const uint32_t p = tile_base + (code & 0x3fffffffu);
-          const Real S = kProdLate ? s1 * get_item<Real, LoadT>(wb.xe, j) : wb.xe[j];
+          const Real S = kProdLate ? rmul(s1, get_item<Real, LoadT>(wb.xe, j)) : wb.xe[j];
           const Real h = intrinsic<Real>(type, K, S);
           const Real hd = qmul(h, d1);
           bool exercise = pre == 1;
@@ -864,7 +945,7 @@ backward_kernel(BwdArgs a) {
             for (int k = 0; k < PPT; ++k) {
               const uint32_t p = p_base + k * kBT;
               if (p < P) {
-                const Real h = payoff<Real>(type, K, sN * (Real)e1[k]);
+                const Real h = payoff<Real>(type, K, rmul(sN, (Real)e1[k]));
                 const Real z = fma(h, dNhi, h * dNlo);
                 euro += (double)z;
                 CHK_ST(a.chk, &Z[p], z);
@@ -896,6 +977,7 @@ backward_kernel(BwdArgs a) {
             cnt += __popc(m);
           }
           __syncwarp();
+#pragma unroll 1
           for (int j0 = 0; j0 < cnt; j0 += 32) {
             const int j = j0 + lane;
             int pre = 0;
@@ -915,7 +997,10 @@ backward_kernel(BwdArgs a) {
             xn += __popc(m);
           }
           __syncwarp();
-          const int full = xn & ~31;
+          // whole warps of items; the last sub-tile takes the remainder too
+          const bool last = sb + 1 == sub || sub_base + TILE0 >= P;
+          const int full = last ? xn : xn & ~31;
+#pragma unroll 1
           for (int j = lane; j < full; j += 32) settle(j);
           const int rem = xn - full;
           Real t0 = (Real)0, t1 = (Real)0;
@@ -934,7 +1019,6 @@ backward_kernel(BwdArgs a) {
           __syncwarp();
           xn = rem;
         }
-        if (lane < xn) settle(lane);  // the items left from the last sub-tile
         // the cash flows stored above are read back by other lanes of the warp
         __threadfence_block();
         __syncwarp();
@@ -1009,12 +1093,26 @@ backward_kernel(BwdArgs a) {
           cnt += __popc(m);
         }
         __syncwarp();
-        Real* t = acc.target();
-        const int full = cnt & ~31;
-        for (int j = lane; j < full; j += 32)
-          accumulate_moments<Real, BASIS, NM>(t, n_itm, get_item<Real, LoadT>(ms, j),
-                                              get_item<Real, LoadT>(mv, j), my[j], xK0, invTh);
-        mcarry = cnt - full;
+        // double: the last sub-tile takes the remainder too (one copy of the
+        // long loop body in the instruction cache)
+        const bool last = kFixed && (sb + 1 == sub || sub_base + TILE0 >= P);
+        const int full = last ? cnt : cnt & ~31;
+        if constexpr (kFixed) {
+#pragma unroll 1
+          for (int j0 = 0; j0 < full; j0 += 32) {
+            const bool have = j0 + lane < full;
+            const int j = have ? j0 + lane : j0;
+            acc.add(s_fix, get_item<Real, LoadT>(ms, j),
+                    BASIS == kBasisSV2 ? get_item<Real, LoadT>(mv, j) : (Real)0, my[j], have, xK0,
+                    invTh);
+            n_itm += have ? 1u : 0u;
+          }
+        } else {
+          Real* t = acc.target();
+          for (int j = lane; j < full; j += 32)
+            accumulate_moments<Real, BASIS, NM>(t, n_itm, ms[j], mv[j], my[j], xK0, invTh);
+        }
+        mcarry = last ? 0 : cnt - full;
         Real r0 = (Real)0, r1 = (Real)0, r2 = (Real)0;
         if (lane < mcarry) {
           r0 = ms[full + lane];
@@ -1028,13 +1126,12 @@ backward_kernel(BwdArgs a) {
           my[lane] = r2;
         }
         __syncwarp();
-        acc.fold();
+        if constexpr (!kFixed) acc.fold();
       }
-      if (mcarry > 0) {  // the carried moment items of the last sub-tile
-        if (lane < mcarry)
-          accumulate_moments<Real, BASIS, NM>(acc.target(), n_itm, get_item<Real, LoadT>(ms, lane),
-                                              get_item<Real, LoadT>(mv, lane), my[lane], xK0,
-                                              invTh);
+      if constexpr (!kFixed) {
+        if (lane < mcarry)  // the carried moment items of the last sub-tile
+          accumulate_moments<Real, BASIS, NM>(acc.target(), n_itm, ms[lane], mv[lane], my[lane],
+                                              xK0, invTh);
         __syncwarp();
       }
     }
@@ -1048,16 +1145,21 @@ backward_kernel(BwdArgs a) {
       sy = warp_sum(sy);
       sy2 = warp_sum(sy2);
     } else if constexpr (!kSingle) {
-      // double: reduce-scatter by recursive halving, all lanes busy (an FP64
-      // warp instruction takes the same pipe time whatever its active
-      // lanes): about NA adds per lane in place of 31 per sum on NA lanes
-      double vs[NA];
-#pragma unroll
-      for (int i = 0; i < NA; ++i) vs[i] = i == 0 ? (double)n_itm : acc.s[i];  // the count: an integer
-      double out;
+      // double: the fixed-point units reduced exactly over the lanes, each
+      // converted by the lane that ends with it
+      using Sums = FixedSums<BASIS>;
+      long long ua[Sums::NU], ub[Sums::NU], oa, ob;
+      acc.units(ua, ub);
       int i;
-      halving_sum<NA, 16>(vs, lane, 0, NA, out, i);
-      if (i >= 0) s_red[warp][i < NM ? i : kSlotRhs + (i - NM)] = out;
+      halving_units<Sums::NU, 16>(ua, ub, lane, 0, Sums::NU, oa, ob, i);
+      const uint32_t items = __reduce_add_sync(0xffffffffu, n_itm);
+      auto slot = [](int u) { return u < NM - 1 ? u + 1 : kSlotRhs + (u - (NM - 1)); };
+      if (i >= 0) s_red[warp][slot(i)] = Sums::value(i, oa, ob, s_fix, type == kPut);
+      if (lane == 0) s_red[warp][0] = (double)items;
+      if (acc.spilled) {  // uniform across the warp
+        __syncwarp();
+        if (lane < Sums::NU) s_red[warp][slot(lane)] += acc.spill;
+      }
     } else {
       // rows per pass: as many as the warp's moment buffers hold
       constexpr int RROWS = (int)(sizeof(wb.m) / (33 * sizeof(float2)));
@@ -1118,11 +1220,12 @@ backward_kernel(BwdArgs a) {
     if (warp == 0) {
       __syncwarp();
       if (tid == 0) {
-        __threadfence();
-        const uint32_t old = atomicAdd(&st->arrive, 1u);
+        // the arrival releases the job's writes and, for the last CTA,
+        // acquires the others'; the next job number is fetched with it
+        const uint32_t old = atom_add_acq_rel_gpu(&st->arrive, 1u);
+        const unsigned long long job = atomicAdd(&a.ctl->next_job, 1ull);
         s_last = (old + 1 == (r + 1) * I.tiles) ? 1 : 0;
-        if (s_last) __threadfence();
-        decode();
+        decode(job);
       }
     }
     __syncthreads();
@@ -1136,6 +1239,7 @@ backward_kernel(BwdArgs a) {
       if (lane < kNSum) {
         double v = 0.0;
         const uint32_t t0 = warp * per, t1 = min(tiles, t0 + per);
+#pragma unroll 8
         for (uint32_t t = t0; t < t1; ++t)
           if (CHK_OK(a.chk, &I.partial[(size_t)t * kNSum + lane], sizeof(double)))
             v += __ldcg(&I.partial[(size_t)t * kNSum + lane]);
@@ -1149,8 +1253,8 @@ backward_kernel(BwdArgs a) {
       }
       __syncthreads();
     }
-    if (tid == 0) {
-      if (final_job) {
+    if (final_job) {
+      if (tid == 0) {
         BwdResult res;
         const double Pd = (double)P;
         const double mean = s_sum[kSlotSumY] / Pd;
@@ -1166,27 +1270,55 @@ backward_kernel(BwdArgs a) {
         res.done = 1;
         CHK_ST(a.chk, &a.results[I.out_index], res);
         if (a.flag_host != nullptr) finish_request(a, I.req);
+      }
+    } else if (!final_job && warp == 0) {
+      double beta = 0.0;  // lane i < 6: coefficient i
+      bool ok;
+      if constexpr (kSerialSolve) {
+        double b6[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+        ok = tid == 0 && solve_normal_equations(NB, s_sum, s_sum + kSlotRhs, b6);
+        ok = __shfl_sync(0xffffffffu, (int)ok, 0) != 0;
+#pragma unroll
+        for (int i = 0; i < 6; ++i) {
+          const double bi = __shfl_sync(0xffffffffu, b6[i], 0);
+          if (lane == i) beta = bi;
+        }
       } else {
-        double beta[6];
-        const bool ok = solve_normal_equations<std::is_same<Real, double>::value>(
-            NB, s_sum, s_sum + kSlotRhs, beta);
+        ok = solve_normal_equations_warp<NB>(s_sum, s_sum + kSlotRhs, lane, beta);
+      }
+      if (!ok) beta = 0.0;
+      if (lane < 6) st->beta[lane] = beta;
+      if (I.beta_hist && lane < 6) {
+        // coefficients in the units of the cash flow discounted to t_n
+        const double to_n = 1.0 / CHK_LD(a.chk, &dtab[n]);
+        CHK_ST(a.chk, &I.beta_hist[(size_t)n * 6 + lane],
+               ok ? (lane < NB ? beta * to_n : 0.0) : __longlong_as_double(0x7ff8000000000000ll));
+      }
+      if (I.beta_z && lane < 7)  // the date's coefficients, kept for an out-of-sample pass
+        CHK_ST(a.chk, &I.beta_z[(size_t)n * 8 + lane], lane < 6 ? beta : (ok ? 1.0 : 0.0));
+      if (lane == 0) {
         if (r == 0) st->euro_sum = s_sum[kSlotEuro];
-        st->itm = __ldcg(&st->itm) + s_sum[0];
-        st->ties = __ldcg(&st->ties) + s_sum[kSlotTies];
-        if (!ok) st->singular = __ldcg(&st->singular) + 1u;
+        // whole numbers: exact in any order
+        atomicAdd(&st->itm, s_sum[0]);
+        atomicAdd(&st->ties, s_sum[kSlotTies]);
+        if (!ok) atomicAdd(&st->singular, 1u);
         st->beta_ok = ok ? 1u : 0u;
-        for (int i = 0; i < 6; ++i) st->beta[i] = ok ? beta[i] : 0.0;
-        if (I.beta_hist) {
-          // coefficients in the units of the cash flow discounted to t_n
-          const double to_n = 1.0 / CHK_LD(a.chk, &dtab[n]);
-          for (int i = 0; i < 6; ++i)
-            CHK_ST(a.chk, &I.beta_hist[(size_t)n * 6 + i],
-                   ok ? (i < NB ? beta[i] * to_n : 0.0) : __longlong_as_double(0x7ff8000000000000ll));
-        }
-        if (I.beta_z) {  // the date's coefficients, kept for an out-of-sample pass
-          for (int i = 0; i < 6; ++i) CHK_ST(a.chk, &I.beta_z[(size_t)n * 8 + i], ok ? beta[i] : 0.0);
-          CHK_ST(a.chk, &I.beta_z[(size_t)n * 8 + 6], ok ? 1.0 : 0.0);
-        }
+      }
+      if (kFixed && lane == 1) {  // the ranges of the next date's fixed-point sums
+        st->range[0] = fix_range(s_sum[2], s_sum[0], 4, 2, s_range[0]);
+        st->range[1] = BASIS == kBasisSV2
+                           ? fix_range(s_sum[mono(0, 2)], s_sum[0], 6, 2, s_range[1])
+                           : s_range[1];
+        st->range[2] = fix_range(s_sum[kSlotRhs], s_sum[0], 4, 1, s_range[2]);
+      }
+    } else if (!final_job && kProdLate && tid == 32) {
+      // beside the solve: the thresholds of the next round's two dates
+      st->thr[0] = s_thrd[1];
+      if (n > 1) st->thr[1] = row_threshold<Real>(type, CHK_LD(a.chk, &stab[n - 1]), I.K);
+    }
+    if (!final_job) {
+      __syncthreads();
+      if (tid == 0) {
         __threadfence();
         st_release_gpu(&st->ready, r + 1);
       }

@@ -219,6 +219,16 @@ template <> struct Draw<float> {
   }
 };
 
+// y ~ 1 / sqrt(a) and the correction: sqrt(a) = g (1 + ep), 1 / sqrt(a) =
+// y (1 + ep), g = a y (0 and 0 for a zero or subnormal a)
+__device__ __forceinline__ void rsqrt_seed(double a, double& y, double& g, double& ep) {
+  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
+  if (__double2hiint(a) < 0x00100000) y = 0.0;
+  g = a * y;
+  const double e = fma(-g, y, 1.0);
+  ep = e * fma(e, 0.375, 0.5);
+}
+
 __device__ __forceinline__ unsigned long long global_timer_ns() {
   unsigned long long t;
   asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
@@ -233,6 +243,13 @@ __device__ __forceinline__ uint32_t ld_acquire_gpu(const uint32_t* p) {
 
 __device__ __forceinline__ void st_release_gpu(uint32_t* p, uint32_t v) {
   asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+}
+
+__device__ __forceinline__ uint32_t atom_add_acq_rel_gpu(uint32_t* p, uint32_t v) {
+  uint32_t old;
+  asm volatile("atom.add.acq_rel.gpu.global.u32 %0, [%1], %2;"
+               : "=r"(old) : "l"(p), "r"(v) : "memory");
+  return old;
 }
 
 __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) {

@@ -28,6 +28,16 @@ __device__ __forceinline__ Real payoff(int type, Real K, Real S) {
 // unnormalised forms for float pairs.
 template <typename R> __device__ __forceinline__ R qmul(R a, R b) { return a * b; }
 template <> __device__ __forceinline__ df qmul<df>(df a, df b) { return mul_nr(a, b); }
+// double: rounded on its own, never contracted into a following sum, so that
+// every kernel and build takes a decision from the same bits
+template <> __device__ __forceinline__ double qmul<double>(double a, double b) {
+  return __dmul_rn(a, b);
+}
+// the normalised product (row value times S multiplier)
+template <typename R> __device__ __forceinline__ R rmul(R a, R b) { return a * b; }
+template <> __device__ __forceinline__ double rmul<double>(double a, double b) {
+  return __dmul_rn(a, b);
+}
 template <typename R> __device__ __forceinline__ void qacc(R& s, R t) { s += t; }
 template <> __device__ __forceinline__ void qacc<df>(df& s, df t) { acc_pair(s, t); }
 // a * b + c
@@ -37,6 +47,9 @@ template <> __device__ __forceinline__ df qfma<df>(df a, df b, df c) {
 }
 template <typename R> __device__ __forceinline__ R qsub(R a, R b) { return a - b; }
 template <> __device__ __forceinline__ df qsub<df>(df a, df b) { return add_sloppy(a, -b); }
+template <> __device__ __forceinline__ double qsub<double>(double a, double b) {
+  return __dsub_rn(a, b);
+}
 // payoff without the max: put K - S, call S - K
 template <typename R>
 __device__ __forceinline__ R intrinsic(int type, R K, R S) {
@@ -67,7 +80,7 @@ template <>
 __device__ __forceinline__ void decide<double>(double hd, double c, bool& exercise, bool& tie) {
   // one FP64 subtraction; sign and exponents compared as integers
   // (2^-33 = 1.16e-10 relative)
-  const double d = hd - c;
+  const double d = __dsub_rn(hd, c);
   const long long bd = __double_as_longlong(d);
   exercise = bd > 0;
   const int ed = (int)((bd >> 52) & 0x7ff);

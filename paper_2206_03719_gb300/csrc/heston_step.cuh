@@ -187,15 +187,6 @@ __device__ __forceinline__ double positive_part(double v) {
   return __double2hiint(v) < 0 ? 0.0 : v;
 }
 
-// y ~ 1 / sqrt(a) and the correction: sqrt(a) = g (1 + ep), 1 / sqrt(a) =
-// y (1 + ep), g = a y (0 and 0 for a zero or subnormal a)
-__device__ __forceinline__ void rsqrt_seed(double a, double& y, double& g, double& ep) {
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  if (__double2hiint(a) < 0x00100000) y = 0.0;
-  g = a * y;
-  const double e = fma(-g, y, 1.0);
-  ep = e * fma(e, 0.375, 0.5);
-}
 __device__ __forceinline__ double rcp_f64(double a) {
   double y;
   asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
