@@ -8,6 +8,7 @@
 
 #include "dfloat.cuh"
 #include "df_tables.h"
+#include "forward_df.h"
 
 namespace lsmc {
 
@@ -16,6 +17,7 @@ struct DfTables {
   float2 qpair[kQPair][kQIntervals];             // G polynomials, pair part
   float qflt[kQDegree + 1 - kQPair][kQIntervals];  // G polynomials, float part
   float qcen[kQIntervals];                       // interval centres
+  DfForward fwd;                                 // quantile segments, 2^(j / kDfExpN)
 };
 
 // Copy the tables into shared memory; the caller synchronises the block.
@@ -26,6 +28,9 @@ __device__ __forceinline__ void load_df_tables(DfTables* t) {
   for (int i = threadIdx.x; i < (kQDegree + 1 - kQPair) * kQIntervals; i += blockDim.x)
     (&t->qflt[0][0])[i] = (&kQCoefFloat[0][0])[i];
   for (int i = threadIdx.x; i < kQIntervals; i += blockDim.x) t->qcen[i] = kQCentre[i];
+  static_assert(sizeof(DfForward) % sizeof(float2) == 0, "copied by pairs");
+  for (int i = threadIdx.x; i < (int)(sizeof(DfForward) / sizeof(float2)); i += blockDim.x)
+    reinterpret_cast<float2*>(&t->fwd)[i] = __ldg(reinterpret_cast<const float2*>(&kDfForward) + i);
 }
 
 // exp(a).  Reduction a = k L + r with L = ln 2 / kExpTab split into three
@@ -60,6 +65,35 @@ __device__ __forceinline__ df exp_df(df a, const float2* tab) {
   const float s = __int_as_float(((k >> 7) + 127) << 23);
   static_assert(kExpTab == 128, "the shift above is log2(kExpTab)");
   return df(__fmul_rn(res.hi, s), __fmul_rn(res.lo, s));
+}
+
+// exp(X ln 2 / kDfExpN) for a log price X in those units: k = rint(X), f =
+// X - k exact; 2^(f / kDfExpN) - 1 by a cubic whose first two terms are pairs
+// (|f ln 2 / kDfExpN| <= 3.4e-4; remainder below 6e-16).  About 38 FP32
+// operations against 45 of exp_df, whose argument is reduced in three parts.
+__device__ __forceinline__ df exp_log_price_df(df X, const DfForward& t) {
+  constexpr float kTop = (float)(88.0 * kDfExpUnit), kBottom = (float)(-87.0 * kDfExpUnit);
+  if (X.hi > kTop) return df(__int_as_float(0x7f800000), 0.0f);
+  if (X.hi < kBottom) return df(0.0f, 0.0f);
+  const float kf = rintf(X.hi);
+  const int k = (int)kf;
+  const df f = two_sum(__fsub_rn(X.hi, kf), X.lo);
+  df p = mul_nr(f, df(kDfExpA1, kDfExpA1Lo));
+  // the quadratic term (up to 6e-8) with its rounding errors
+  const df f2 = two_prod(f.hi, f.hi);
+  const float t2 = __fmul_rn(f2.hi, kDfExpA2);
+  float e2 = __fmaf_rn(f2.hi, kDfExpA2, -t2);
+  e2 = __fmaf_rn(f2.lo, kDfExpA2, __fmaf_rn(f2.hi, kDfExpA2Lo, e2));
+  e2 = __fmaf_rn(__fmul_rn(f2.hi, f.hi), kDfExpA3, e2);
+  const float pl = p.lo;
+  p = quick_two_sum(p.hi, t2);
+  p.lo = __fadd_rn(p.lo, __fadd_rn(pl, e2));
+  const float2 tj = t.exp2[k & (kDfExpN - 1)];
+  const df q = mul_nr(df(tj.x, tj.y), p);
+  const df s = quick_two_sum(tj.x, q.hi);
+  const df res = quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(tj.y, q.lo)));
+  const float sc = __int_as_float(((k >> kDfExpNLog2) + 127) << 23);
+  return df(__fmul_rn(res.hi, sc), __fmul_rn(res.lo, sc));
 }
 
 // exp(x) in double, table-driven (Tang's method): k = rint(x 128 / ln 2)
@@ -144,13 +178,42 @@ __device__ __forceinline__ df normal_quantile_lower_df(df p, const DfTables* t) 
 // With M = 2m + 1 = hi 2^21 + l21 (l21 odd, < 2^21): u = hi 2^-32 + l21 2^-53
 // and 1 - u = (~hi) 2^-32 + (2^21 - l21) 2^-53, both exact before pairing.
 template <> struct Draw<df> {
+  // Phi^-1 of the grid point of words (hi, lo): the lower tail min(u, 1 - u),
+  // its octave, segment and t in [-1/2, 1/2) by integer work as in
+  // Draw<double>::quantile, t as two floats; the segment's polynomial in
+  // float down to t^3 and in pairs below (about 35 FP32 operations).  Beyond the
+  // tabulated octaves normal_quantile_lower_df, with which every draw went
+  // before (normcdfinvf and a Halley step with an exponential, some 200).
   __device__ __forceinline__ static df quantile(uint32_t hi, uint32_t lo,
-                                                const DfTables* t) {
-    const uint32_t l21 = (lo >> 11) | 1u;
-    const bool upper = (hi >> 31) != 0u;
-    const df p = upper ? uniform_pair(~hi, 0x200000u - l21) : uniform_pair(hi, l21);
-    const df z = normal_quantile_lower_df(p, t);
-    return upper ? -z : z;
+                                                const DfTables* tab) {
+    const uint32_t s = (uint32_t)((int)hi >> 31);
+    const uint32_t ph = hi ^ s;
+    const uint32_t pl = ((lo ^ s) & 0xfffff000u) | 0x800u;
+    df z;
+    if (ph >= (0x80000000u >> kQsOct)) {
+      const DfForward& d = tab->fwd;
+      const int k = __clz((int)ph);
+      const uint32_t nh = __funnelshift_l(pl, ph, k), nl = pl << k;
+      const int j = (k << 6) + (int)(nh >> 25) - 128;
+      const float t = __uint_as_float(0x3f800000u | ((nh & 0x1ffffffu) >> 2)) - 1.5f;
+      const float tl = __fmul_rn(
+          __uint_as_float(0x3f800000u | ((nh & 3u) << 21) | (nl >> 11)) - 1.0f, 0x1p-23f);
+      const float2 c2 = d.qp[2][j], c1 = d.qp[1][j], c0 = d.qp[0][j];
+      const float f = __fmaf_rn(__fmaf_rn(d.qf[2][j], t, d.qf[1][j]), t, d.qf[0][j]);
+      df g = quick_two_sum(c2.x, __fmul_rn(f, t));
+      g.lo = __fadd_rn(g.lo, c2.y);
+      df p = two_prod(g.hi, t);
+      p.lo = __fmaf_rn(g.hi, tl, __fmaf_rn(g.lo, t, p.lo));
+      df h = quick_two_sum(c1.x, p.hi);
+      h.lo = __fadd_rn(h.lo, __fadd_rn(c1.y, p.lo));
+      p = two_prod(h.hi, t);
+      p.lo = __fmaf_rn(h.hi, tl, __fmaf_rn(h.lo, t, p.lo));
+      z = two_sum(c0.x, p.hi);
+      z = quick_two_sum(z.hi, __fadd_rn(z.lo, __fadd_rn(c0.y, p.lo)));
+    } else {
+      z = normal_quantile_lower_df(uniform_pair(ph, pl >> 11), tab);
+    }
+    return s ? -z : z;
   }
   __device__ __forceinline__ static void make(uint4 w, df& u, df& omu, df& zV, df& zX,
                                               const DfTables* t) {

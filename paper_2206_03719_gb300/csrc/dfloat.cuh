@@ -137,6 +137,11 @@ __device__ __forceinline__ df add_sloppy(df a, df b) {
   return quick_two_sum(s.hi, __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo)));
 }
 
+// a b + c for inner loops: unnormalised product, sloppy sum
+__device__ __forceinline__ df madd_df(df a, df b, df c) { return add_sloppy(mul_nr(a, b), c); }
+__device__ __forceinline__ df twice_df(df a) { return df(a.hi + a.hi, a.lo + a.lo); }
+__device__ __forceinline__ df half_df(df a) { return df(0.5f * a.hi, 0.5f * a.lo); }
+
 // Running sum of pairs: two-sum of the high parts, the low parts collected
 // unnormalised (renormalise with quick_two_sum before using the total).
 __device__ __forceinline__ void acc_pair(df& s, df t) {
@@ -148,6 +153,19 @@ __device__ __forceinline__ void acc_pair(df& s, df t) {
 // x * 2^k, exact
 __device__ __forceinline__ df ldexp_df(df a, int k) {
   return df(ldexpf(a.hi, k), ldexpf(a.lo, k));
+}
+
+// y ~ 1 / sqrt(a) from the special-function unit and what corrects it:
+// sqrt(a) = (g + gl) (1 + ep), 1 / sqrt(a) = y (1 + ep), g = RN(a.hi y),
+// ep from the residual 1 - a y^2 (2^-22) to second order, within 2^-46.
+// All zero for a.hi = 0.
+__device__ __forceinline__ void rsqrt_seed_df(df a, float& y, float& g, float& gl, float& ep) {
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(a.hi));
+  if (!(a.hi >= 1.17549435e-38f)) y = 0.0f;
+  g = __fmul_rn(a.hi, y);
+  gl = __fmaf_rn(a.lo, y, __fmaf_rn(a.hi, y, -g));
+  const float e = __fmaf_rn(-gl, y, __fmaf_rn(-g, y, 1.0f));
+  ep = __fmul_rn(e, __fmaf_rn(e, 0.375f, 0.5f));
 }
 
 __device__ __forceinline__ df sqrt_df(df a) {

@@ -218,12 +218,20 @@ forward_kernel(FwdArgs a) {
     // and the per-group state lives in shared memory
     __shared__ Real xs[kMaxGroups][kFwdBlock], vs[kMaxGroups][kFwdBlock];
     const int t = threadIdx.x;
+    bool scaled = false;  // plans have unit row scale
+    for (int g = 0; g < ng; ++g)
+      scaled = scaled || gc[g].out_scale.hi != 1.0f || gc[g].out_scale.lo != 0.0f;
+    auto row_value = [&](const GroupConst<Real>& c, Real xg, Real vg) {
+      const Real e = Fm<Real>::exp_(log_price<Real, SCHEME>(c, xg, vg), tabs);
+      return narrow<St>(scaled ? c.out_scale * e : e);
+    };
     for (int g = 0; g < ng; ++g) {
       const GroupConst<Real>& c = gc[g];
-      xs[g][t] = ck_index ? CHK_LD(a.chk, &c.CX[ck_index * c.ld + p]) : (Real)0;
+      xs[g][t] = ck_index ? CHK_LD(a.chk, &c.CX[ck_index * c.ld + p])
+                          : log_price_start<Real, SCHEME>(c);
       vs[g][t] = ck_index ? CHK_LD(a.chk, &c.CV[ck_index * c.ld + p]) : c.v0;
       if (first_row) {
-        CHK_ST(a.chk, &((St*)c.E)[p], narrow<St>(c.out_scale * Fm<Real>::exp_(xs[g][t], tabs)));
+        CHK_ST(a.chk, &((St*)c.E)[p], row_value(c, xs[g][t], vs[g][t]));
         if (c.V)
           CHK_ST(a.chk, &((St*)c.V)[p],
                  narrow<St>((SCHEME == kSchemeFT && vs[g][t] < (Real)0) ? (Real)0 : vs[g][t]));
@@ -246,7 +254,7 @@ forward_kernel(FwdArgs a) {
         vs[g][t] = vg;
         if (store_rows) {
           const size_t off = (size_t)(n + 1 - row0) * c.ld + p;
-          CHK_ST(a.chk, &((St*)c.E)[off], narrow<St>(c.out_scale * Fm<Real>::exp_(xg, tabs)));
+          CHK_ST(a.chk, &((St*)c.E)[off], row_value(c, xg, vg));
           if (c.V)
             CHK_ST(a.chk, &((St*)c.V)[off],
                    narrow<St>((SCHEME == kSchemeFT && vg < (Real)0) ? (Real)0 : vg));
@@ -398,7 +406,7 @@ __global__ void exp_kernel(const Real* __restrict__ x, Real* __restrict__ y, siz
   const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n) return;
   if constexpr (std::is_same<Real, double>::value) y[i] = exp_f64(x[i]);
-  else if constexpr (kPair) y[i] = Fm<df>::exp_(x[i], tabs);
+  else if constexpr (kPair) y[i] = exp_df(x[i], tabs->exp2);
   else y[i] = Fm<float>::exp_(x[i], nullptr);
 }
 

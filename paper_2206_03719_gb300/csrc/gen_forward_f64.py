@@ -1,5 +1,5 @@
-"""Write forward_f64.h: the tables of the double-precision forward pass,
-computed in 40-digit arithmetic with mpmath.
+"""Write forward_f64.h and forward_df.h: the tables of the double-precision and
+float-pair forward passes, computed in 40-digit arithmetic with mpmath.
 
     python paper_2206_03719_gb300/csrc/gen_forward_f64.py
 
@@ -13,21 +13,26 @@ to double one after another from the lowest up.  Stored coefficient-major
 Exponential: 2^(j / EXPN), j = 0..EXPN-1, and the coefficients of
 2^(f / EXPN) - 1 on |f| <= 1/2 (Taylor to f^3, the f^4 term economised onto
 f^2).
+
+Float pairs: the same segments at degree 5 (c_0..c_2 as pairs, the others as
+floats) and 2^(j / EXPN_DF) as pairs.
 """
 import os
 
 import mpmath as mp
+import numpy as np
 
 mp.mp.dps = 40
 OCT, SEG, DEG = 10, 64, 6
 EXPN = 2048
+DEG_DF, EXPN_DF = 5, 1024
 
 
 def quantile(p):
     return -mp.sqrt(2) * mp.erfinv(1 - 2 * p)
 
 
-def segment(k, i):
+def segment(k, i, DEG=DEG):
     """coefficients of the segment's polynomial in t, and its error"""
     left = mp.mpf(2) ** -(k + 1) * (1 + mp.mpf(i) / SEG)
     width = mp.mpf(2) ** -(k + 1) / SEG
@@ -38,7 +43,10 @@ def segment(k, i):
         for j in range(DEG + 1):
             A[r, j] = t ** j
         b[r] = quantile(left + width * (t + mp.mpf(0.5)))
-    c = [float(x) for x in mp.lu_solve(A, b)]
+    sol = mp.lu_solve(A, b)
+    if DEG == DEG_DF:
+        return list(sol), 0.0
+    c = [float(x) for x in sol]
     worst = mp.mpf(0)
     for s in (-0.5, -0.37, -0.2, 0.0, 0.11, 0.3, 0.45, 0.5):
         v = mp.mpf(0)
@@ -90,5 +98,53 @@ def main():
         f.write("    },\n};\n\n}  // namespace lsmc\n")
 
 
+def pair(x):
+    """(hi, lo) floats of an mp value"""
+    hi = np.float32(float(x))
+    return hi, np.float32(float(mp.mpf(x) - mp.mpf(float(hi))))
+
+
+def main_df():
+    rows = [[] for _ in range(DEG_DF + 1)]
+    for k in range(1, OCT + 1):
+        for i in range(SEG):
+            for j, c in enumerate(segment(k, i, DEG_DF)[0]):
+                rows[j].append(c)
+    L = mp.log(2) / EXPN_DF
+    here = os.path.dirname(os.path.abspath(__file__))
+    with open(os.path.join(here, "forward_df.h"), "w") as f:
+        f.write("// forward_df.h -- written by gen_forward_f64.py (40-digit mpmath); do not edit.\n"
+                "#pragma once\n\nnamespace lsmc {\n\n"
+                "constexpr int kDfExpN = %d, kDfExpNLog2 = %d;\n"
+                "constexpr double kDfExpUnit = %.17e;  // kDfExpN / ln 2\n"
+                "constexpr float kDfExpA1 = %.9ef, kDfExpA1Lo = %.9ef;\n"
+                "constexpr float kDfExpA2 = %.9ef, kDfExpA2Lo = %.9ef, kDfExpA3 = %.9ef;\n\n"
+                "struct DfForward {\n"
+                "  float2 qp[3][%d];  // quantile segments: c_0, c_1, c_2 as pairs\n"
+                "  float qf[%d][%d];   // c_3, c_4, c_5\n"
+                "  float2 exp2[kDfExpN];  // 2^(j / kDfExpN)\n"
+                "};\n\n" % ((EXPN_DF, EXPN_DF.bit_length() - 1, float(1 / L)) + pair(L) +
+                            pair(L ** 2 / 2) + (float(L ** 3 / 6), OCT * SEG, DEG_DF - 2, OCT * SEG)))
+        f.write("static __device__ const DfForward kDfForward = {\n    {\n")
+        f2 = lambda x: "{%.9ef, %.9ef}" % pair(x)  # noqa: E731
+        for r in rows[:3]:
+            f.write("        {\n")
+            for i in range(0, len(r), 4):
+                f.write("            " + " ".join(f2(v) + "," for v in r[i:i + 4]) + "\n")
+            f.write("        },\n")
+        f.write("    },\n    {\n")
+        for r in rows[3:]:
+            f.write("        {\n")
+            for i in range(0, len(r), 6):
+                f.write("            " + " ".join("%.9ef," % float(v) for v in r[i:i + 6]) + "\n")
+            f.write("        },\n")
+        f.write("    },\n    {\n")
+        for i in range(0, EXPN_DF, 4):
+            f.write("        " + " ".join(f2(mp.mpf(2) ** (mp.mpf(j) / EXPN_DF)) + ","
+                                          for j in range(i, i + 4)) + "\n")
+        f.write("    },\n};\n\n}  // namespace lsmc\n")
+
+
 if __name__ == "__main__":
     main()
+    main_df()

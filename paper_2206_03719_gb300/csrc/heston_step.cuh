@@ -29,18 +29,19 @@ template <typename Real> __device__ __forceinline__ void load_tables(Tab<Real>* 
       reinterpret_cast<double2*>(t)[i] = __ldg(&src[i]);
   }
 }
-// The kernels' dynamic shared memory above 48 KB needs an opt-in.
+// The kernels' shared memory above 48 KB (static and dynamic) needs an opt-in.
 template <auto Kernel> static cudaError_t allow_dynamic(size_t bytes) {
-  if (bytes <= 40 * 1024) return cudaSuccess;
+  if (bytes == 0) return cudaSuccess;
   return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
 }
 
 // The unit of a path's log price x: double keeps x in units of
-// ln 2 / kExpN, so that its exponential needs no argument reduction (k is x
+// ln 2 / kExpN (float pairs ln 2 / kDfExpN), so that its exponential needs no argument reduction (k is x
 // rounded to an integer, exactly); the constants that x is made of are
 // converted once per group, with the unit as a pair.
 template <typename Real> __device__ __forceinline__ double in_log_units(double c) {
-  return std::is_same<Real, double>::value ? fma(kExpUnit, c, kExpUnitLo * c) : c;
+  if (std::is_same<Real, double>::value) return fma(kExpUnit, c, kExpUnitLo * c);
+  return std::is_same<Real, df>::value ? kDfExpUnit * c : c;
 }
 
 // exp(X ln 2 / kExpN) for a log price X in those units: k = rint(X), f = X - k
@@ -79,13 +80,14 @@ template <> struct Fm<df> {
   __device__ static df div(df a, df b) { return a / b; }
   __device__ static df sqrt_(df a) { return sqrt_df(a); }
   __device__ static df log_(df a, const DfTables* t) { return log_df(a, t->exp2); }
-  __device__ static df exp_(df a, const DfTables* t) { return exp_df(a, t->exp2); }
+  __device__ static df exp_(df a, const DfTables* t) { return exp_log_price_df(a, t->fwd); }
 };
 
 template <typename Real>
 struct GroupConst {
-  // QE: m = mA + mB v, s^2 = sA + sB v (double: half of it), x1 = x + c0 +
-  // K1 v + K2 v1 + sqrt(K3 (v + v1)) Z; in double the state is x - K2 v, K1
+  // QE: m = mA + mB v, s^2 = sA + sB v, x1 = x + c0 + K1 v + K2 v1 +
+  // sqrt(K3 (v + v1)) Z.  In double and float pairs sA + sB v is half of s^2,
+  // the state is x - K2 v, K1
   // holds K1 + K2 (x - K2 v moves by c0 + (K1 + K2) v + sqrt(...) Z: K1 and K2
   // are large and nearly cancel, and their rounding errors would grow with the
   // steps), and c0, K1, K2, K3, mudt, hdt,
@@ -105,7 +107,7 @@ struct GroupConst {
 // with gamma1 = gamma2 = 1/2; the plain Euler coefficients for FT).
 template <typename Real>
 __device__ void make_group_const(const FwdGroup& g, GroupConst<Real>& c) {
-  constexpr bool kDouble = std::is_same<Real, double>::value;
+  constexpr bool kWide = !std::is_same<Real, float>::value;  // double, float pairs
   auto u = [](double x) { return in_log_units<Real>(x); };
   const double dt = g.dt, k = g.kappa, th = g.theta, xi = g.xi, rho = g.rho;
   const double E = exp(-k * dt);
@@ -113,12 +115,12 @@ __device__ void make_group_const(const FwdGroup& g, GroupConst<Real>& c) {
   c.mA = (Real)(th * omE);
   c.mB = (Real)E;
   if (xi > 0.0) {
-    const double half = kDouble ? 0.5 : 1.0;
+    const double half = kWide ? 0.5 : 1.0;
     c.sB = (Real)(half * (xi * xi * E * omE / k));
     c.sA = (Real)(half * (th * xi * xi * omE * omE / (2.0 * k)));
     const double K0 = -rho * k * th * dt / xi;
     const double h = 0.5 * dt * (k * rho / xi - 0.5);
-    c.K1 = (Real)(kDouble ? u(2.0 * h) : u(h - rho / xi));
+    c.K1 = (Real)(kWide ? u(2.0 * h) : u(h - rho / xi));
     c.K2 = (Real)u(h + rho / xi);
     c.c0 = (Real)u((g.r - g.q) * dt + K0);
   } else {
@@ -275,6 +277,70 @@ __device__ __forceinline__ void qe_core<double>(double mA, double mB, double sA,
   v = v1;
 }
 
+// ---- float pairs ----------------------------------------------------------------
+// the variance step of the scheme's definition (means outside the range where
+// the products below keep their low words)
+static __device__ __noinline__ df qe_variance_plain(df m, df h2, df omu, df zV,
+                                                    const DfTables* t) {
+  const df s2 = twice_df(h2), m2 = m * m;
+  if (s2 <= mul_f(m2, 1.5f)) {
+    const df inv = twice_df(m2) / s2;
+    const df tt = inv - df(1.0f, 0.0f);
+    const df b2 = tt + sqrt_df(inv * tt);
+    const df q = sqrt_df(b2) + zV;
+    return m / (df(1.0f, 0.0f) + b2) * q * q;
+  }
+  const df omp = twice_df(m2) / (s2 + m2);
+  return omu >= omp ? df(0.0f, 0.0f) : m / omp * log_df(omp / omu, t->exp2);
+}
+
+// The step in the form of qe_core<double>: about 190 FP32 operations with the
+// quadratic branch where the direct form took 380 (a pair's division is 25, its
+// full addition 20, a product with a sum that cannot cancel 15).
+template <>
+__device__ __forceinline__ void qe_core<df>(df mA, df mB, df sA, df sB, df c0, df K1, df K2, df K3,
+                                            df& x, df& v, df omu, df zV, df zX,
+                                            const DfTables* t) {
+  const df m = madd_df(mB, v, mA);
+  const df h2 = madd_df(sB, v, sA);
+  df v1;
+  if (m.hi > 1e-6f && m.hi < 1e6f) {
+    const df A = mul_nr(m, m);
+    const df D = add_sloppy(A, -h2);
+    // psi <= 3/2  <=>  3 D >= h2
+    if (__fadd_rn(__fmaf_rn(3.0f, D.hi, -h2.hi), __fmaf_rn(3.0f, D.lo, -h2.lo)) >= 0.0f) {
+      float y, g, gl, ep;
+      rsqrt_seed_df(D, y, g, gl, ep);
+      const df d = quick_two_sum(g, __fmaf_rn(g, ep, gl)), r(y, __fmul_rn(y, ep));
+      const df n = mul_nr(h2, d);
+      const df X = mul_nr(n, add_sloppy(m, d));
+      rsqrt_seed_df(quick_two_sum(X.hi, X.lo), y, g, gl, ep);
+      df s = two_prod(n.hi, y);  // n / sqrt(X)
+      s.lo = __fmaf_rn(s.hi, ep, __fmaf_rn(n.lo, y, s.lo));
+      const df q = madd_df(s, zV, d);
+      v1 = mul_nr(mul_nr(q, q), r);
+      v1 = quick_two_sum(v1.hi, v1.lo);
+    } else {
+      const df B = add_sloppy(A, twice_df(h2)), A2 = twice_df(quick_two_sum(A.hi, A.lo));
+      const df bu = B * omu;
+      if (bu >= A2) {
+        v1 = df(0.0f, 0.0f);
+      } else {
+        const df R = df(1.0f, 0.0f) / (bu * m);
+        v1 = half_df(B) * (R * bu) * log_df(A2 * (R * m), t->exp2);
+      }
+    }
+  } else {
+    v1 = qe_variance_plain(m, h2, omu, zV, t);
+  }
+  const df w = mul_nr(K3, add_sloppy(v, v1));
+  float y, g, gl, ep;
+  rsqrt_seed_df(quick_two_sum(w.hi, w.lo), y, g, gl, ep);
+  const df sq = quick_two_sum(g, __fmaf_rn(g, ep, gl));
+  x = add_sloppy(x, add_sloppy(mul_nr(sq, zX), madd_df(K1, v, c0)));
+  v = v1;
+}
+
 template <typename Real>
 __device__ __forceinline__ void qe_step(const GroupConst<Real>& c, Real& x, Real& v,
                                         Real omu, Real zV, Real zX, const Tab<Real>* t) {
@@ -285,12 +351,14 @@ __device__ __forceinline__ void qe_step(const GroupConst<Real>& c, Real& x, Real
 // of a state x with variance v.
 template <typename Real, int SCHEME>
 __device__ __forceinline__ Real log_price_start(const GroupConst<Real>& c) {
-  if constexpr (std::is_same<Real, double>::value && SCHEME == kSchemeQE) return -c.K2 * c.v0;
+  if constexpr (!std::is_same<Real, float>::value && SCHEME == kSchemeQE) return -(c.K2 * c.v0);
   else return (Real)0;
 }
 template <typename Real, int SCHEME>
 __device__ __forceinline__ Real log_price(const GroupConst<Real>& c, Real x, Real v) {
   if constexpr (std::is_same<Real, double>::value && SCHEME == kSchemeQE) return fma(c.K2, v, x);
+  else if constexpr (std::is_same<Real, df>::value && SCHEME == kSchemeQE)
+    return madd_df(c.K2, v, x);
   else return x;
 }
 
@@ -315,6 +383,18 @@ __device__ __forceinline__ void ft_step<double>(const GroupConst<double>& c, dou
   const double sq = fma(g, ep, g);
   const double v1 = fma(c.xi, sq * zV, fma(c.kdt, c.theta - vp, v));
   x = x + fma(-c.hdt, vp, c.mudt) + sq * fma(c.rhob, zX, c.rho * zV);
+  v = v1;
+}
+
+template <>
+__device__ __forceinline__ void ft_step<df>(const GroupConst<df>& c, df& x, df& v, df zV, df zX) {
+  const df vp = v.hi > 0.0f ? v : df(0.0f, 0.0f);
+  float y, g, gl, ep;
+  rsqrt_seed_df(vp * c.dt, y, g, gl, ep);
+  const df sq = quick_two_sum(g, __fmaf_rn(g, ep, gl));
+  const df v1 = (v + mul_nr(c.kdt, c.theta - vp)) + mul_nr(c.xi, sq * zV);
+  const df shock = mul_nr(sq, madd_df(c.rhob, zX, mul_nr(c.rho, zV)));
+  x = x + add_sloppy(shock, madd_df(-c.hdt, vp, c.mudt));
   v = v1;
 }
 

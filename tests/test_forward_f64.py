@@ -1,5 +1,5 @@
-"""The double-precision stepper's tables and step (forward_f64.h, Draw<double>
-and qe_core<double>): the quantile segments and the exponential's cubic against
+"""The double-precision and float-pair steppers' tables and steps (forward_f64.h,
+forward_df.h, Draw and qe_core): the quantile segments and the exponential's cubic against
 40-digit values on the CPU; the draws and the paths of the GPU at the models
 where the step changes form."""
 import os
@@ -118,3 +118,30 @@ def test_paths_where_the_step_changes_form_match_oracle(kw):
     # oracle's own rounding is amplified by the step: 1e-13 absolute
     assert np.allclose(V.cpu().numpy(), Vo, rtol=1e-11,
                        atol=1e-13 if model["theta"] > 1e-10 else 1e-84)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("kw", [
+    dict(xi=2.5, kappa=0.3, theta=0.02), dict(v0=0.0),
+    dict(v0=1e-8, theta=1e-8, xi=1e-4),            # means outside the range of the products
+    dict(rho=1.0), dict(rho=-1.0),
+], ids=lambda k: ",".join("%s=%g" % i for i in k.items()))
+def test_pair_paths_where_the_step_changes_form_match_oracle(kw):
+    from gpu_common import torch_cuda
+    from paper_2206_03719_gb300 import build
+    from paper_2206_03719_gb300 import lsmc as L
+    torch = torch_cuda()
+    build.build()
+    model = dict(S0=100.0, r=0.02, q=0.0, v0=0.04, kappa=1.5, theta=0.04, xi=0.3, rho=-0.7)
+    model.update(kw)
+    P, N = 500, 30
+    S = torch.empty((N + 1, P, 2), dtype=torch.float32, device="cuda")
+    V = torch.empty_like(S)
+    L.lsmc_paths(L.lsmc_heston(**model), 0.5, L.LSMC_SCHEME_QE, L.LSMC_DF, P, N, 5, 2,
+                 S.data_ptr(), V.data_ptr())
+    So, Vo = oracle.paths(oracle.heston(**model), 0.5, oracle.QE, P, N, 5, 2)
+    # the stage tests' tolerances for pairs; at xi = 2.5 the step amplifies a
+    # rounding 2^-48 as it does 2^-53 in double (1e-13 there): 1e-11
+    atol = 1e-11 if model["xi"] > 1 else 1e-14 * max(1.0, model["theta"] / 0.04)
+    assert np.allclose(S.double().sum(-1).cpu().numpy(), So, rtol=1e-11, atol=0)
+    assert np.allclose(V.double().sum(-1).cpu().numpy(), Vo, rtol=1e-10, atol=atol)
