@@ -140,6 +140,13 @@ __device__ __forceinline__ double norm_quantile_f64(double u, double omu) {
   return x * r;
 }
 
+// A normal float as a double by integer operations (the conversion instruction
+// runs on the FP64 pipe); zero and subnormals give some value below 2^-125.
+__device__ __forceinline__ double widen_float(float f) {
+  const int b = __float_as_int(f);
+  return __hiloint2double(((b >> 3) & (int)0x8fffffff) + (896 << 20), b << 29);
+}
+
 // Tables of a working precision's draws and steps, staged in shared memory by
 // the kernels that step paths (the index differs from lane to lane): double
 // the quantile segments and powers of two of forward_f64.h, float pairs those
@@ -165,15 +172,17 @@ template <> struct Draw<double> {
            (1.0 - 0x1p-53);
   }
   // Phi^-1 of the grid point of words (hi, lo).  FP64 operations bound the
-  // double-precision stepper (18 clocks a warp on an SM, an integer operation
-  // half a clock, a gathered shared-memory load 4.5), so everything but the
-  // polynomial is integer work: the lower tail p = min(u, 1 - u) as the
-  // 64-bit word p 2^64, its octave by a leading-zero count, the segment from
-  // the next six bits, and t in [-1/2, 1/2) from the remaining (at most 52)
-  // bits put into a mantissa; then a degree-6 polynomial of the segment: 7
-  // FP64 operations, against 45 of norm_quantile_f64, which stays for the
-  // tails beyond the tabulated octaves (p < 2^-11, a tenth of a percent).
-  // Within 2.5e-16 of Phi^-1, max(1, |z|) relative.
+  // double-precision stepper (18 clocks a warp on an SM, an integer or FP32
+  // operation a third to half a clock, a gathered shared-memory load 4.5), so
+  // only the last sum is in double: the lower tail p = min(u, 1 - u) is the
+  // 64-bit word p 2^64, its octave a leading-zero count, the segment the
+  // next six bits, t in [-1/2, 1/2) the remaining (at most 46) bits as two
+  // floats; the segment's degree-6 polynomial without its constant runs in
+  // floats down to t^4 and in float pairs below (its value is at most 2^-6 of
+  // the quantile's scale, so 46 bits of it suffice).  2 FP64 operations;
+  // norm_quantile_f64's 45 remain for the tails beyond the tabulated octaves
+  // (p < 2^-11, a tenth of a percent).  Within 3e-16 of Phi^-1, max(1, |z|)
+  // relative.
   __device__ __forceinline__ static double quantile(uint32_t hi, uint32_t lo,
                                                     const F64Tables* tab) {
     const uint32_t s = (uint32_t)((int)hi >> 31);  // all ones in the upper half
@@ -184,12 +193,25 @@ template <> struct Draw<double> {
       const int k = __clz((int)ph);  // p in [2^-(k + 1), 2^-k)
       const uint32_t nh = __funnelshift_l(pl, ph, k), nl = pl << k;
       const int j = (k << 6) + (int)(nh >> 25) - 128;  // (k - 1) 64 + segment
-      const double t = __hiloint2double((int)(0x3ff00000u | ((nh & 0x1ffffffu) >> 5)),
-                                        (int)__funnelshift_r(nl, nh, 5)) -
-                       1.5;
-      z = tab->qc[kQsDeg][j];
+      const float t = __uint_as_float(0x3f800000u | ((nh & 0x1ffffffu) >> 2)) - 1.5f;
+      const float tl = __fmul_rn(
+          __uint_as_float(0x3f800000u | ((nh & 3u) << 21) | (nl >> 11)) - 1.0f, 0x1p-23f);
+      const float f = __fmaf_rn(__fmaf_rn(tab->qf[2][j], t, tab->qf[1][j]), t, tab->qf[0][j]);
+      const float2 c3 = tab->qp[2][j];
+      df g = quick_two_sum(c3.x, __fmul_rn(f, t));
+      g.lo = __fadd_rn(g.lo, c3.y);
+      df p;
 #pragma unroll
-      for (int i = kQsDeg - 1; i >= 0; --i) z = fma(z, t, tab->qc[i][j]);
+      for (int i = 1; i >= 0; --i) {
+        const float2 c = tab->qp[i][j];
+        p = two_prod(g.hi, t);
+        p.lo = __fmaf_rn(g.hi, tl, __fmaf_rn(g.lo, t, p.lo));
+        g = quick_two_sum(c.x, p.hi);
+        g.lo = __fadd_rn(g.lo, __fadd_rn(c.y, p.lo));
+      }
+      p = two_prod(g.hi, t);
+      p.lo = __fmaf_rn(g.hi, tl, __fmaf_rn(g.lo, t, p.lo));
+      z = tab->q0[j] + (widen_float(p.hi) + widen_float(p.lo));
     } else {
       const double p = grid_point(ph, pl & 0xfffff000u);
       z = norm_quantile_f64(p, 1.0 - p);
@@ -220,13 +242,33 @@ template <> struct Draw<float> {
 };
 
 // y ~ 1 / sqrt(a) and the correction: sqrt(a) = g (1 + ep), 1 / sqrt(a) =
-// y (1 + ep), g = a y (0 and 0 for a zero or subnormal a)
+// y (1 + ep), g = a y (y = g = 0 for a zero, subnormal or negative a).  Two
+// FP64 operations: the special-function unit's seed (2^-22) is improved to
+// 2^-40 in FP32 on a's mantissa m 4^q (m in [1, 4) as two floats) and put
+// into a double by integer operations, so the correction ep = (1 - a y^2) / 2
+// is needed to first order only.
 __device__ __forceinline__ void rsqrt_seed(double a, double& y, double& g, double& ep) {
-  asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(a));
-  if (__double2hiint(a) < 0x00100000) y = 0.0;
+  const int hi = __double2hiint(a);
+  const uint32_t lo = (uint32_t)__double2loint(a);
+  const int q = (hi - (1023 << 20)) >> 21;
+  const float m = __uint_as_float(__funnelshift_l(lo, (uint32_t)(hi - (q << 21) - (896 << 20)), 3));
+  const float ml = __fmul_rn(__uint_as_float(0x3f800000u | ((lo & 0x1fffffffu) >> 6)) - 1.0f,
+                             __int_as_float((__float_as_int(m) & 0x7f800000) - (23 << 23)));
+  float yf;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(m));
+  // inside (1/2, 1): the integer sum below then stays in one binade
+  yf = fminf(fmaxf(yf, 0.5f + 0x1p-21f), 1.0f - 0x1p-24f);
+  const float p = __fmul_rn(yf, yf), pe = __fmaf_rn(yf, yf, -p);
+  const float r = __fmaf_rn(-ml, p, __fmaf_rn(-m, pe, __fmaf_rn(-m, p, 1.0f)));
+  const float c = __fmul_rn(yf, __fmul_rn(r, __fmaf_rn(r, 0.375f, 0.5f)));
+  const long long d = (long long)__float2int_rn(__fmul_rn(c, 0x1p49f)) << 4;
+  const int b = __float_as_int(yf);
+  const long long bits =
+      (((long long)((b >> 3) + (896 << 20)) << 32) | (long long)(uint32_t)(b << 29)) + d;
+  const int yh = (int)(bits >> 32) - (q << 20);
+  y = hi < 0x00100000 ? 0.0 : __hiloint2double(yh, (int)bits);
   g = a * y;
-  const double e = fma(-g, y, 1.0);
-  ep = e * fma(e, 0.375, 0.5);
+  ep = fma(-g, __hiloint2double(yh - (1 << 20), (int)bits), 0.5);
 }
 
 __device__ __forceinline__ unsigned long long global_timer_ns() {

@@ -44,20 +44,40 @@ template <typename Real> __device__ __forceinline__ double in_log_units(double c
   return std::is_same<Real, df>::value ? kDfExpUnit * c : c;
 }
 
-// exp(X ln 2 / kExpN) for a log price X in those units: k = rint(X), f = X - k
-// exact, 2^(f / kExpN) - 1 by a cubic (|f ln 2 / kExpN| <= 1.7e-4; remainder
-// below 5e-18), times 2^(k / kExpN) from the table and the exponent: 7 FP64
-// operations against 10 of exp_f64 (a table of 128 and a two-part reduction).
-// Beyond |x| = 354 CUDA's exp.
+// exp(X ln 2 / kExpN) for a log price X in those units.  X is split by integer
+// operations into k = rint(X) and f = X - k to 44 bits; 2^(f / kExpN) - 1
+// (at most 1.7e-4, so float pairs carry it past the double's last bit) by a
+// cubic with f in units of 2^-22, its first two terms in pairs; times
+// 2^(k / kExpN) from the table and the exponent: 2 FP64 operations and about
+// 50 integer and FP32 ones, against 10 FP64 of exp_f64.  Beyond |x| = 177
+// CUDA's exp.
 __device__ __forceinline__ double exp_log_price(double X, const F64Tables* tab) {
-  if ((__double2hiint(X) & 0x7fffffff) >= ((1023 + 20) << 20)) return exp(X * kExpUnitInv);
-  const double magic = 6755399441055744.0;  // 1.5 * 2^52: k in the low word
-  const double t = X + magic;
-  const int k = __double2loint(t);
-  const double f = X - (t - magic);
-  const double p = fma(fma(f, kExpA3, kExpA2), f, kExpA1) * f;
+  const int hi = __double2hiint(X), mag = hi & 0x7fffffff;
+  if (mag >= ((1023 + 19) << 20)) return exp(X * kExpUnitInv);
+  const uint32_t lo = (uint32_t)__double2loint(X);
+  // |X| 2^44: the mantissa shifted left by 11 and right by 1042 - exponent
+  const uint32_t mh = ((uint32_t)mag & 0xfffffu) | 0x100000u;
+  const unsigned long long m =
+      ((unsigned long long)__funnelshift_l(lo, mh, 11) << 32) | (lo << 11);
+  unsigned long long u;
+  asm("shr.u64 %0, %1, %2;" : "=l"(u) : "l"(m), "r"(1042 - (mag >> 20)));
+  const long long s = (long long)(hi >> 31);
+  const long long R = ((long long)u ^ s) - s + (1ll << 43);
+  const int k = (int)(R >> 32) >> 12;
+  const float f = __uint_as_float(0x4b000000u | (__funnelshift_r((uint32_t)R, (uint32_t)(R >> 32),
+                                                                 22) & 0x3fffffu)) -
+                  (8388608.0f + 2097152.0f);
+  const float fl = __uint_as_float(0x3f800000u | (((uint32_t)R & 0x3fffffu) << 1)) - 1.0f;
+  df p = two_prod(f, kExpA1);
+  float e = __fmaf_rn(fl, kExpA1, __fmaf_rn(f, kExpA1Lo, p.lo));
+  const df f2 = two_prod(f, f);
+  const float t2 = __fmul_rn(f2.hi, kExpA2);
+  e = __fadd_rn(e, __fmaf_rn(f2.hi, kExpA2, -t2));
+  e = __fmaf_rn(__fmaf_rn(f + f, fl, f2.lo), kExpA2, __fmaf_rn(f2.hi, kExpA2Lo, e));
+  e = __fmaf_rn(__fmul_rn(f2.hi, f), kExpA3, e);
+  p = quick_two_sum(p.hi, t2);
   const double T = tab->exp2[k & (kExpN - 1)];
-  const double y = fma(T, p, T);
+  const double y = fma(T, widen_float(p.hi) + widen_float(__fadd_rn(p.lo, e)), T);
   return __hiloint2double(__double2hiint(y) + ((k >> kExpNLog2) << 20), __double2loint(y));
 }
 
@@ -179,10 +199,9 @@ __device__ __forceinline__ void qe_core(Real mA, Real mB, Real sA, Real sB, Real
 // ---- double precision --------------------------------------------------------
 // An FP64 instruction holds the pipe of an SM for 18 clocks a warp on GB300;
 // CUDA's square root and division are eight of them each (142 clocks).  The
-// special-function unit's 20-bit seeds take 2 clocks, so square roots and
-// quotients are formed here from a seed y and one third-order correction
-// (the binomial series of (1 - e)^-1/2 and (1 - e)^-1 to e^2, e ~ 2^-20, the
-// remainder below 2^-59), sharing what can be shared.
+// special-function unit's seeds take 2 clocks, so square roots are formed from
+// rsqrt_seed (its seed improved in FP32) and quotients from a seed y and one
+// third-order correction (e ~ 2^-20), sharing what can be shared.
 
 // max(v, 0) of a double, the sign read as an integer
 __device__ __forceinline__ double positive_part(double v) {
@@ -217,15 +236,15 @@ static __device__ __noinline__ double qe_variance_plain(double m, double h2, dou
 
 // Andersen QE step in double.  With h2 = s^2 / 2 and d = sqrt(m^2 - h2) the
 // quadratic branch's a and b are a = m - d = h2 / (m + d) and a b^2 = d, so
-//   v1 = a (b + Z)^2 = (d + sqrt(a d) Z)^2 / d,
-//   sqrt(a d) = h2 d / sqrt(h2 d (m + d)),
-// two reciprocal square roots (the first giving d and 1 / d) in place of two
-// square roots and two divisions.  Exponential branch: with A = m^2,
+//   v1 = a (b + Z)^2 = d (1 + w)^2,  w = sqrt(a / d) Z,
+//   sqrt(a / d) = h2 / sqrt(h2 (d m + d^2)),
+// two reciprocal square roots in place of two square roots and two divisions.  Exponential branch: with A = m^2,
 // B = A + 2 h2: 1 - p = 2 A / B and 1 / beta = B / (2 m), and one reciprocal
 // of B U m (U = 1 - U_V) gives both quotients of v1 = B / (2 m) log(2 A / (B U)).
-// About 33 FP64 operations with the quadratic branch against 60 before (the
-// FP64 forward pass of the 131,072 x 252 book 27.5 -> 14.3 ms with the
-// table quantile and exponential).
+// 26 FP64 operations with the quadratic branch and the exponential against 70
+// before (the
+// FP64 forward pass of the 131,072 x 252 book 27.5 -> 14.3 ms with the table
+// quantile and exponential, -> 11.5 with what can be in FP32 moved there).
 template <>
 __device__ __forceinline__ void qe_core<double>(double mA, double mB, double sA, double sB,
                                                 double c0, double K1, double K2, double K3,
@@ -248,13 +267,11 @@ __device__ __forceinline__ void qe_core<double>(double mA, double mB, double sA,
     if (quad) {
       double y, g, ep;
       rsqrt_seed(D, y, g, ep);
-      const double d = fma(g, ep, g), r = fma(y, ep, y);
-      const double n = h2 * d;
-      double y2, g2, ep2;
-      rsqrt_seed(n * (m + d), y2, g2, ep2);
-      const double ny = n * y2;
-      const double sz = fma(ny, ep2, ny) * zV, q = d + sz;
-      v1 = positive_part(fma(q, sz * r, q));  // q^2 / d with sz / d = q / d - 1
+      const double d = fma(g, ep, g);
+      rsqrt_seed(h2 * fma(d, m, D), y, g, ep);
+      const double hy = h2 * y;
+      const double w = fma(hy, ep, hy) * zV, q = fma(d, w, d);
+      v1 = positive_part(fma(q, w, q));
     } else {
       const double A = m * m, B = fma(2.0, h2, A), bu = B * omu;
       // 2 A and B / 2 by their exponents
@@ -272,8 +289,7 @@ __device__ __forceinline__ void qe_core<double>(double mA, double mB, double sA,
   }
   double y, g, ep;
   rsqrt_seed(K3 * (v + v1), y, g, ep);
-  const double gz = g * zX;
-  x = x + (fma(gz, ep, fma(K1, v, c0)) + gz);
+  x = x + fma(fma(g, ep, g), zX, fma(K1, v, c0));
   v = v1;
 }
 
@@ -311,15 +327,15 @@ __device__ __forceinline__ void qe_core<df>(df mA, df mB, df sA, df sB, df c0, d
     if (__fadd_rn(__fmaf_rn(3.0f, D.hi, -h2.hi), __fmaf_rn(3.0f, D.lo, -h2.lo)) >= 0.0f) {
       float y, g, gl, ep;
       rsqrt_seed_df(D, y, g, gl, ep);
-      const df d = quick_two_sum(g, __fmaf_rn(g, ep, gl)), r(y, __fmul_rn(y, ep));
-      const df n = mul_nr(h2, d);
-      const df X = mul_nr(n, add_sloppy(m, d));
+      const df d = quick_two_sum(g, __fmaf_rn(g, ep, gl));
+      const df X = mul_nr(h2, madd_df(d, m, D));
       rsqrt_seed_df(quick_two_sum(X.hi, X.lo), y, g, gl, ep);
-      df s = two_prod(n.hi, y);  // n / sqrt(X)
-      s.lo = __fmaf_rn(s.hi, ep, __fmaf_rn(n.lo, y, s.lo));
-      const df q = madd_df(s, zV, d);
-      v1 = mul_nr(mul_nr(q, q), r);
-      v1 = quick_two_sum(v1.hi, v1.lo);
+      df w = two_prod(h2.hi, y);  // h2 / sqrt(X)
+      w.lo = __fmaf_rn(w.hi, ep, __fmaf_rn(h2.lo, y, w.lo));
+      w = mul_nr(w, zV);
+      const df q = madd_df(d, w, d);
+      v1 = madd_df(q, w, q);
+      if (v1.hi < 0.0f) v1 = df(0.0f, 0.0f);
     } else {
       const df B = add_sloppy(A, twice_df(h2)), A2 = twice_df(quick_two_sum(A.hi, A.lo));
       const df bu = B * omu;
