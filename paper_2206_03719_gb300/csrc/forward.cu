@@ -270,13 +270,18 @@ forward_kernel(FwdArgs a) {
 
 // ---- STAC-A2 multi-asset path reduction (Sec. 2.2.1, Sec. 4.1) ---------------
 // M[n][p] = max over assets of S_a[n][p].  Like the paper's loop interchange,
-// the assets are the outer loop of a thread (KA of them at a time, their
-// state in registers and their steps interleaved), the dates the inner
-// loop, and the running maximum lives in M itself (read, compared, written
-// back by the one thread that owns the path).  Element (path, asset, date)
-// draws from Philox counter (path, date, stream, asset); the common
-// log-price shock of (path, date), used when the assets are correlated,
-// from counter (path, date, stream, 0xFFFFFFFF).
+// the assets are outside the dates; here a CTA takes 128 paths and KA assets
+// (their state in registers, their steps interleaved) through all dates and
+// adds its running maxima to M by atomic maxima on the values' bits (positive
+// numbers order like their bits), M starting as a negative NaN.  One CTA per
+// 128 paths over all assets, M read and written back by the thread that owns
+// the path, left the chip uneven where paths are few: 25,000 paths are 196
+// CTAs on 152 SMs, and the SMs with two of them decide (10 assets x 126 dates
+// in double 4.60 ms, 3.17 split in pairs of assets; 30 x 100 x 1,000 paths
+// 20.3 -> 0.59).
+// Element (path, asset, date) draws from Philox counter (path, date, stream,
+// asset); the common log-price shock of (path, date), used when the assets are
+// correlated, from counter (path, date, stream, 0xFFFFFFFF).
 
 template <typename Real>
 __device__ __forceinline__ Real common_shock(uint4 w, const Tab<Real>* t);
@@ -294,32 +299,51 @@ __device__ __forceinline__ df common_shock<df>(uint4 w, const DfTables* t) {
   return Draw<df>::quantile(w.z, w.w, t);
 }
 
-// fmax; for the non-negative doubles here by their bits (an FP64 comparison
-// costs the pipe as much as a multiply-add), a NaN giving the other operand
-template <typename Real> __device__ __forceinline__ Real larger(Real a, Real b) {
-  return fmax(a, b);
+// The bits of a value as a signed integer that orders like the value; NaNs
+// (and the initial state, all ones) below every number, so that a maximum
+// passes them over as fmax does.  A pair's low word is mapped so that it
+// orders as an unsigned integer; unmap_pairs_kernel undoes it.
+__device__ __forceinline__ long long max_key(double v) {
+  const long long b = __double_as_longlong(v);
+  return b > 0x7ff0000000000000ll ? -1ll : b;
 }
-template <> __device__ __forceinline__ double larger<double>(double a, double b) {
-  const long long inf = 0x7ff0000000000000ll;
-  const long long ka = __double_as_longlong(a), kb = __double_as_longlong(b);
-  if (ka > inf) return b;
-  return kb > ka && kb <= inf ? b : a;
+__device__ __forceinline__ int max_key(float v) {
+  const int b = __float_as_int(v);
+  return b > 0x7f800000 ? -1 : b;
+}
+__device__ __forceinline__ long long max_key(df v) {
+  const int b = __float_as_int(v.hi);
+  if (b > 0x7f800000 || b < 0) return -1ll;
+  const uint32_t l = __float_as_uint(v.lo);
+  return ((long long)b << 32) | (l ^ ((uint32_t)((int)l >> 31) | 0x80000000u));
+}
+
+__global__ void unmap_pairs_kernel(uint2* __restrict__ m, size_t n CHK_PARAM) {
+  const size_t i = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n) return;
+  uint2 v = CHK_LD(chk, &m[i]);  // x: low word, y: the high word's bits
+  const uint32_t l = (v.x & 0x80000000u) ? v.x ^ 0x80000000u : ~v.x;
+  v.x = v.y;
+  v.y = l;
+  CHK_ST(chk, &m[i], v);
 }
 
 template <typename Real, int SCHEME, int KA>
 __global__ void __launch_bounds__(kFwdBlock)
 multi_max_kernel(MultiArgs a) {
-  __shared__ GroupConst<Real> gc[kMaxAssets];
+  using Key = typename std::conditional<std::is_same<Real, float>::value, int, long long>::type;
+  __shared__ GroupConst<Real> gc[KA];
   extern __shared__ __align__(16) unsigned char tab_raw[];
   Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
   load_tables<Real>(tabs);
   const double dt = a.T / (double)a.N;
-  for (uint32_t i = threadIdx.x; i < a.n_assets; i += blockDim.x) {
-    const MultiModel& m = a.assets[i];
+  const uint32_t a0 = blockIdx.y * KA;
+  if (threadIdx.x < KA && a0 + threadIdx.x < a.n_assets) {
+    const MultiModel& m = a.assets[a0 + threadIdx.x];
     FwdGroup g{};
     g.v0 = m.v0; g.kappa = m.kappa; g.theta = m.theta; g.xi = m.xi; g.rho = m.rho;
     g.r = m.r; g.q = m.q; g.dt = dt; g.out_scale = m.S0;
-    make_group_const<Real>(g, gc[i]);
+    make_group_const<Real>(g, gc[threadIdx.x]);
   }
   __syncthreads();
   const uint32_t p = blockIdx.x * kFwdBlock + threadIdx.x;
@@ -327,56 +351,82 @@ multi_max_kernel(MultiArgs a) {
   const uint2 key = make_uint2((uint32_t)a.seed, (uint32_t)(a.seed >> 32));
   const bool corr = a.sqrt_rho > 0.0;
   const Real sr = (Real)a.sqrt_rho, s1r = (Real)a.sqrt_1m_rho;
-  Real* M = (Real*)a.M;
+  Key* M = (Key*)a.M;
   const size_t P = a.P;
+  const int na = (int)min((uint32_t)KA, a.n_assets - a0);
 
-  for (uint32_t a0 = 0; a0 < a.n_assets; a0 += KA) {
-    Real x[KA], v[KA];
-    Real m0 = (Real)0;
+  Real x[KA], v[KA];
+  Key k0 = -1;
+#pragma unroll
+  for (int k = 0; k < KA; ++k) {
+    const GroupConst<Real>& c = gc[k < na ? k : 0];
+    x[k] = log_price_start<Real, SCHEME>(c);
+    v[k] = c.v0;
+    const Key s0 = max_key(c.out_scale);
+    k0 = s0 > k0 ? s0 : k0;
+  }
+  // one CTA row has all the assets: plain stores
+  const bool split = gridDim.y > 1;
+  auto put = [&](Key* q, Key k) {
+    if (!CHK_OK(a.chk, q, sizeof(Key))) return;
+    if (split) atomicMax(q, k);
+    else *q = k;
+  };
+  put(&M[p], k0);
+  for (uint32_t n = 0; n < a.N; ++n) {
+    Real zc = (Real)0;
+    if (corr)
+      zc = common_shock<Real>(philox4x32_10(make_uint4(p, n, a.stream_id, 0xFFFFFFFFu), key),
+                              tabs);
+    Key mx = -1;
 #pragma unroll
     for (int k = 0; k < KA; ++k) {
-      const uint32_t ai = a0 + k < a.n_assets ? a0 + k : a0;
-      x[k] = log_price_start<Real, SCHEME>(gc[ai]);
-      v[k] = gc[ai].v0;
-      if (k == 0 || gc[ai].out_scale > m0) m0 = gc[ai].out_scale;
-    }
-    CHK_ST(a.chk, &M[p], a0 == 0 ? m0 : fmax(CHK_LD(a.chk, &M[p]), m0));
-    for (uint32_t n = 0; n < a.N; ++n) {
-      Real zc = (Real)0;
-      if (corr)
-        zc = common_shock<Real>(philox4x32_10(make_uint4(p, n, a.stream_id, 0xFFFFFFFFu), key),
-                                tabs);
-      Real mx = (Real)0;
-#pragma unroll
-      for (int k = 0; k < KA; ++k) {
-        if (a0 + k < a.n_assets) {
-          const GroupConst<Real>& c = gc[a0 + k];
-          const uint4 w = philox4x32_10(make_uint4(p, n, a.stream_id, a0 + k), key);
-          Real u, omu, zV, zX;
-          Draw<Real>::make(w, u, omu, zV, zX, tabs);
-          if (corr) zX = sr * zc + s1r * zX;
-          if (SCHEME == kSchemeQE) {
-            qe_step<Real>(c, x[k], v[k], omu, zV, zX, tabs);
-          } else {
-            ft_step<Real>(c, x[k], v[k], zV, zX);
-          }
-          const Real S = c.out_scale * Fm<Real>::exp_(log_price<Real, SCHEME>(c, x[k], v[k]), tabs);
-          mx = k == 0 ? S : larger(mx, S);
+      if (k < na) {
+        const GroupConst<Real>& c = gc[k];
+        const uint4 w = philox4x32_10(make_uint4(p, n, a.stream_id, a0 + k), key);
+        Real u, omu, zV, zX;
+        Draw<Real>::make(w, u, omu, zV, zX, tabs);
+        if (corr) zX = sr * zc + s1r * zX;
+        if (SCHEME == kSchemeQE) {
+          qe_step<Real>(c, x[k], v[k], omu, zV, zX, tabs);
+        } else {
+          ft_step<Real>(c, x[k], v[k], zV, zX);
         }
+        const Real S = c.out_scale * Fm<Real>::exp_(log_price<Real, SCHEME>(c, x[k], v[k]), tabs);
+        const Key s = max_key(S);
+        mx = s > mx ? s : mx;
       }
-      const size_t off = (size_t)(n + 1) * P + p;
-      CHK_ST(a.chk, &M[off], a0 == 0 ? mx : larger(CHK_LD(a.chk, &M[off]), mx));
     }
+    put(&M[(size_t)(n + 1) * P + p], mx);
   }
 }
 
+template <typename Real, int SCHEME, int KA>
+static cudaError_t launch_multi_k(const MultiArgs& a, cudaStream_t s) {
+  const dim3 grid((a.P + kFwdBlock - 1) / kFwdBlock, (a.n_assets + KA - 1) / KA);
+  const size_t cells = (size_t)(a.N + 1) * a.P;
+  cudaError_t e = allow_dynamic<multi_max_kernel<Real, SCHEME, KA>>(tab_bytes<Real>());
+  if (e == cudaSuccess && grid.y > 1) e = cudaMemsetAsync(a.M, 0xFF, cells * sizeof(Real), s);
+  if (e != cudaSuccess) return e;
+  multi_max_kernel<Real, SCHEME, KA><<<grid, kFwdBlock, tab_bytes<Real>(), s>>>(a);
+  e = cudaGetLastError();
+  if constexpr (std::is_same<Real, df>::value) {
+    if (e != cudaSuccess) return e;
+    unmap_pairs_kernel<<<(unsigned)((cells + kBlock - 1) / kBlock), kBlock, 0, s>>>(
+        (uint2*)a.M, cells CHK_ARG(a.chk));
+    e = cudaGetLastError();
+  }
+  return e;
+}
+
+// Two assets a CTA; in single precision four where the paths alone give every
+// SM a few dozen CTAs (fewer maxima per date: 3 assets x 60 dates x 1,000,000
+// paths 1.01 ms with two, 0.98 with four; float pairs 4.50 and 5.63).
 template <typename Real, int SCHEME>
 static cudaError_t launch_multi_s(const MultiArgs& a, cudaStream_t s) {
-  const unsigned blocks = (a.P + kFwdBlock - 1) / kFwdBlock;
-  const cudaError_t e = allow_dynamic<multi_max_kernel<Real, SCHEME, 4>>(tab_bytes<Real>());
-  if (e != cudaSuccess) return e;
-  multi_max_kernel<Real, SCHEME, 4><<<blocks, kFwdBlock, tab_bytes<Real>(), s>>>(a);
-  return cudaGetLastError();
+  if constexpr (std::is_same<Real, float>::value)
+    if (a.P >= (1u << 19)) return launch_multi_k<Real, SCHEME, 4>(a, s);
+  return launch_multi_k<Real, SCHEME, 2>(a, s);
 }
 
 template <typename Real>
@@ -388,8 +438,22 @@ static cudaError_t launch_multi_t(const MultiArgs& a, int scheme, cudaStream_t s
 cudaError_t launch_multi_max(const MultiArgs& a, int precision, int scheme, cudaStream_t s) {
   if (a.P == 0 || a.N == 0 || a.n_assets == 0) return cudaSuccess;
   if (precision == kPrecFP64) return launch_multi_t<double>(a, scheme, s);
-  if (precision == kPrecDF) return launch_multi_t<df>(a, scheme, s);
-  return launch_multi_t<float>(a, scheme, s);
+  if (precision == kPrecMixed) return launch_multi_t<float>(a, scheme, s);
+  if (((uintptr_t)a.M & 7u) == 0) return launch_multi_t<df>(a, scheme, s);
+  // pairs of floats at an address that is not a multiple of 8: the 64-bit
+  // maxima run on an aligned copy
+  const size_t bytes = (size_t)(a.N + 1) * a.P * sizeof(df);
+  MultiArgs b = a;
+  cudaError_t e = cudaMallocAsync(&b.M, bytes, s);
+  if (e != cudaSuccess) return e;
+#ifdef LSMC_CHECKED
+  b.chk.lo[0] = (unsigned long long)b.M;
+  b.chk.hi[0] = b.chk.lo[0] + bytes;
+#endif
+  e = launch_multi_t<df>(b, scheme, s);
+  if (e == cudaSuccess) e = cudaMemcpyAsync(a.M, b.M, bytes, cudaMemcpyDeviceToDevice, s);
+  const cudaError_t f = cudaFreeAsync(b.M, s);
+  return e == cudaSuccess ? f : e;
 }
 
 // The exponential of a log price (the E rows are S0 exp(x)): exp_f64 in

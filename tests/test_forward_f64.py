@@ -150,3 +150,45 @@ def test_pair_paths_where_the_step_changes_form_match_oracle(kw):
     atol = 1e-11 if model["xi"] > 1 else 1e-14 * max(1.0, model["theta"] / 0.04)
     assert np.allclose(S.double().sum(-1).cpu().numpy(), So, rtol=1e-11, atol=0)
     assert np.allclose(V.double().sum(-1).cpu().numpy(), Vo, rtol=1e-10, atol=atol)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("A,P", [(1, 130), (2, 1), (3, 257), (5, 128)])
+def test_reduction_in_pairs_of_assets_is_the_maximum_of_the_assets(A, P):
+    # single precision and pairs: the maximum over separately reduced assets,
+    # bit for bit (one asset per call cannot be: each draws by its index, so
+    # the reduction over the first k assets grows with k); and pairs at an
+    # address that is not a multiple of 8
+    from gpu_common import torch_cuda
+    from paper_2206_03719_gb300 import build, workloads
+    from paper_2206_03719_gb300 import lsmc as L
+    torch = torch_cuda()
+    build.build()
+    N = 7
+    models = [L.lsmc_heston(**m) for m in workloads.stac_models(A)]
+
+    def run(ms, prec, offset=0):
+        n = (N + 1) * P * (2 if prec == L.LSMC_DF else 1)
+        dt = torch.float64 if prec == L.LSMC_FP64 else torch.float32
+        buf = torch.full((n + 1,), float("nan"), dtype=dt, device="cuda")
+        M = buf[offset:offset + n]
+        L.lsmc_multi_asset_max(ms, 0.5, L.LSMC_SCHEME_QE, prec, 0.0, P, N, 3, 1, M.data_ptr())
+        torch.cuda.synchronize()
+        return M.cpu().numpy().copy()
+
+    for prec in (L.LSMC_FP64, L.LSMC_MIXED, L.LSMC_DF):
+        got = run(models, prec)
+        assert np.all(np.isfinite(got))
+        if prec == L.LSMC_DF:
+            assert np.array_equal(got, run(models, prec, 1))
+            got = got.reshape(-1, 2).astype(np.float64).sum(-1)
+        for k in range(1, A):
+            part = run(models[:k], prec)
+            if prec == L.LSMC_DF:
+                part = part.reshape(-1, 2).astype(np.float64).sum(-1)
+            assert np.all(got >= part)
+        ref = oracle.multi_max([oracle.heston(**m) for m in workloads.stac_models(A)], 0.5,
+                               oracle.QE, P, N, 3, 1,
+                               grid=oracle.GRID_F32 if prec == L.LSMC_MIXED else oracle.GRID_F64)
+        rtol = {L.LSMC_FP64: 1e-12, L.LSMC_DF: 1e-11, L.LSMC_MIXED: 1e-3}[prec]
+        assert np.allclose(got.reshape(N + 1, P), ref, rtol=rtol, atol=0)
