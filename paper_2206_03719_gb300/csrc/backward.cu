@@ -502,6 +502,7 @@ backward_kernel(BwdArgs a) {
   constexpr int NA = NM + NB;                         // register sums
   constexpr int TILE0 = kBT * PPT;
   constexpr int NW = kBT / 32;
+  constexpr int kTaker = 32;                          // the thread that takes jobs
 
   __shared__ JobInfo s_job;
   __shared__ uint32_t s_cum[kCumTab];
@@ -540,14 +541,15 @@ backward_kernel(BwdArgs a) {
   // threshold on the stored value), so the compaction buffers hold the
   // stored value and S = s e is formed on the dense lists, where no lane idles
   constexpr bool kProdLate = kCompact;
-  // Job decoding by thread 0.  A job number is taken when the CTA has arrived
-  // with its previous job (only once the CTA can start it).  Job numbers only
+  // Job decoding by one thread (kTaker, in another warp than the arrival).  A
+  // job number is taken when the CTA arrives with its previous job (only once
+  // the CTA can start it).  Job numbers only
   // grow, so the round is found from the last one's; the instance by a binary
   // search over every s_step-th entry of cum_tiles in shared memory (dependent
   // global loads here were on the path of every job).  An error recorded by
   // another CTA is seen in the wait for the previous date.
   const uint32_t cum_step = (a.n_inst + kCumTab - 1) / kCumTab;
-  uint32_t round = 0;                          // thread 0: the last job's round,
+  uint32_t round = 0;                             // kTaker: the last job's round,
   unsigned long long round_lo = 0, round_hi = 0;  // its first job and the next round's
   auto decode = [&](unsigned long long job) {
     JobInfo ji;
@@ -592,7 +594,7 @@ backward_kernel(BwdArgs a) {
   for (uint32_t i = tid; i * cum_step < a.n_inst; i += kBT)
     s_cum[i] = CHK_LD(a.chk, &a.cum_tiles[i * cum_step]);
   __syncthreads();
-  if (tid == 0) {
+  if (tid == kTaker) {
     // the round of the first job: the last one with round_off <= job
     const unsigned long long job = atomicAdd(&a.ctl->next_job, 1ull);
     uint32_t lo = 0, hi = a.n_rounds;
@@ -629,6 +631,23 @@ backward_kernel(BwdArgs a) {
     const uint32_t sub = I.sub;
     const uint32_t tile_base = ji.tile * (sub * TILE0);
 
+    // small jobs: their rows on the way to L1 while the CTA waits
+    if (sub <= 2) {
+      const ptrdiff_t q1 = ((ptrdiff_t)n + 1 - (ptrdiff_t)a.row0) * (ptrdiff_t)ld;
+#pragma unroll
+      for (int k = 0; k < PPT; ++k) {
+        const uint32_t p = tile_base + k * kBT + tid;
+        if (p < P && !final_job) {
+          prefetch_l1(&E[q1 - (ptrdiff_t)ld + p]);
+          prefetch_l1(&E[q1 + p]);
+          if (BASIS == kBasisSV2) {
+            prefetch_l1(&V[q1 - (ptrdiff_t)ld + p]);
+            prefetch_l1(&V[q1 + p]);
+          }
+        }
+      }
+    }
+
     // ---- warp 0: wait for the exercise rule of date n + 1, then convert the
     // per-job constants to the working precision once, a constant per lane ----
     if (warp == 0) {
@@ -658,10 +677,10 @@ backward_kernel(BwdArgs a) {
         const unsigned long long t0 = global_timer_ns();
         unsigned spins = 0, ns = 32;
         while (ld_acquire_gpu(&st->ready) < r) {
-          // back off (32 ns doubling to 512 ns); the error word and the
+          // back off (32 ns doubling to poll_ns); the error word and the
           // clock are read every 32nd time
           __nanosleep(ns);
-          ns = ns < 512 ? 2 * ns : 512;
+          ns = min(2 * ns, a.poll_ns);
           if ((++spins & 31) == 0) {
             if (ld_volatile(&a.ctl->error) != 0) { ok = 0; break; }
             if (spins > (1u << 26) || global_timer_ns() - t0 > a.timeout_ns) {
@@ -1217,16 +1236,17 @@ backward_kernel(BwdArgs a) {
     // the partial was written by warp 0 alone and every other write of this
     // job is ordered before the reduction barrier above, so a warp-level
     // sync suffices before the fence and the arrival
+    // meanwhile another warp takes the next job
     if (warp == 0) {
       __syncwarp();
       if (tid == 0) {
         // the arrival releases the job's writes and, for the last CTA,
-        // acquires the others'; the next job number is fetched with it
+        // acquires the others'
         const uint32_t old = atom_add_acq_rel_gpu(&st->arrive, 1u);
-        const unsigned long long job = atomicAdd(&a.ctl->next_job, 1ull);
         s_last = (old + 1 == (r + 1) * I.tiles) ? 1 : 0;
-        decode(job);
       }
+    } else if (tid == kTaker) {
+      decode(atomicAdd(&a.ctl->next_job, 1ull));
     }
     __syncthreads();
     if (!s_last) continue;
@@ -1317,11 +1337,9 @@ backward_kernel(BwdArgs a) {
       if (n > 1) st->thr[1] = row_threshold<Real>(type, CHK_LD(a.chk, &stab[n - 1]), I.K);
     }
     if (!final_job) {
+      // the barrier orders the CTA's writes before the release
       __syncthreads();
-      if (tid == 0) {
-        __threadfence();
-        st_release_gpu(&st->ready, r + 1);
-      }
+      if (tid == 0) st_release_gpu(&st->ready, r + 1);
     }
     __syncthreads();
   }

@@ -196,6 +196,19 @@ int sm_count(lsmc_ctx* ctx) {
   return n > 0 ? n : 1;
 }
 
+// CTAs of a backward launch over rounds [r0, r1): the resident ones, but no
+// more than the jobs of two consecutive rounds (or 64: CTAs that start early
+// have read their tables when their turn comes).  A job waits for the round
+// before its own, so CTAs beyond that only poll, and what they poll is the
+// line on which the others arrive (4096 x 32, five regressions of 16 tiles:
+// 13.0 us a date with 1216 CTAs, 11.8 with 160).
+int backward_grid(const PlanLayout& L, uint64_t cap, size_t r0, size_t r1) {
+  uint64_t most = std::min<uint64_t>(64, L.round_off[r1] - L.round_off[r0]);
+  for (size_t r = r0; r < r1; ++r)
+    most = std::max<uint64_t>(most, L.round_off[std::min(r + 2, r1)] - L.round_off[r]);
+  return (int)std::max<uint64_t>(1, std::min<uint64_t>(cap, most));
+}
+
 // Device layout of a plan: tables | state + control | results | out |
 // scale tables | partials | Y | paths.
 int plan_bind_and_upload(lsmc_plan* p, void* ext_S, void* ext_V, double* beta_hist) {
@@ -281,6 +294,9 @@ int plan_bind_and_upload(lsmc_plan* p, void* ext_S, void* ext_V, double* beta_hi
   p->fa.next_job_value = 0;
   p->fa.stream_xor = 0;
   p->fa.store_fmt = L.opt.store;
+  p->fa.max_groups = 1;
+  for (const auto& c : L.contracts) p->fa.max_groups = std::max(p->fa.max_groups, c.n_groups);
+  p->fa.sms = (uint32_t)sm_count(p->ctx);
   // one seed for every contract: the Philox round keys as kernel parameters
   p->fa.uniform_key = 0;
   if (!L.contracts.empty()) {
@@ -320,7 +336,9 @@ int plan_bind_and_upload(lsmc_plan* p, void* ext_S, void* ext_V, double* beta_hi
   p->ba.n_inst = (uint32_t)L.inst.size();
   const int occ = occupancy(p->ctx, prec, L.opt.basis, plan_ppt(L.opt), L.opt.store);
   const uint64_t cap = (uint64_t)occ * sm_count(p->ctx);
-  p->bwd_grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(cap, L.total_jobs));
+  p->bwd_grid = backward_grid(L, cap, 0, L.active.size());
+  // few CTAs poll without disturbing the arrivals; a full grid backs off
+  p->ba.poll_ns = (uint64_t)p->bwd_grid * 4 <= cap ? 64 : 512;
   p->h_out.resize(L.greeks.size());
   p->h_res.resize(L.n_results);
 #ifdef LSMC_CHECKED
@@ -450,8 +468,9 @@ uint64_t tune_key(const lsmc_request* reqs, size_t n, const PlanOptions& o) {
 }
 
 // Backward shape of a plan: autotuned if this kind of launch was tuned, else
-// the precision's paths per thread and about four jobs per resident CTA in
-// the busiest round; overrides (tuning sweeps) win.
+// the precision's paths per thread and the sub-tiles of least estimated cost
+// (single precision: about four jobs per resident CTA in the busiest round);
+// overrides (tuning sweeps) win.
 void choose_shape(lsmc_ctx* ctx, const lsmc_request* reqs, size_t n, PlanOptions* o) {
   uint32_t tuned = 0;
   if (ctx) {
@@ -464,6 +483,16 @@ void choose_shape(lsmc_ctx* ctx, const lsmc_request* reqs, size_t n, PlanOptions
   const uint32_t ctas = (uint32_t)occupancy(ctx, o->precision, o->basis, ppt, o->store) *
                         (uint32_t)sm_count(ctx);
   o->sub = choose_sub(reqs, n, o->precision, ppt, ctas);
+  const bool fixed = (tuned & 0xffffu) || (ctx && ctx->sub_override);
+  if (o->precision != LSMC_MIXED && !fixed) {
+    // a plan of few jobs: each request's shape from itself, so that a small
+    // book's results are those of its requests priced alone, bit for bit
+    if (o->sub == 1 && n > 1)
+      for (size_t i = 0; i < n; ++i)
+        o->sub_req.push_back(choose_sub_cost(reqs + i, 1, o->precision, ppt, ctas));
+    else
+      o->sub = choose_sub_cost(reqs, n, o->precision, ppt, ctas);
+  }
   if (tuned & 0xffffu) o->sub = tuned & 0xffffu;
   if (ctx && ctx->sub_override) o->sub = ctx->sub_override;
 }
@@ -547,7 +576,8 @@ int plan_enqueue(lsmc_plan* p, bool timed = false) {
         BwdArgs b = p->ba;
         b.row0 = d0;
         b.total_jobs = j1;
-        const int grid = (int)std::max<uint64_t>(1, std::min<uint64_t>(cap, j1 - j0));
+        const int grid = backward_grid(p->L, cap, std::min<uint64_t>(r_lo, nr),
+                                       std::min<uint64_t>((uint64_t)r_hi + 1, nr));
         LSMC_CUDA(launch_backward(b, prec, p->L.opt.basis, plan_ppt(p->L.opt), grid, p->stream));
       }
     }
@@ -1494,6 +1524,11 @@ static int stage_plan(const lsmc_heston* m, double T, int32_t scheme, int32_t pr
   int rc = plan_options(nullptr, &q, 1, &o);
   if (rc) return rc;
   o.raw_paths = true;
+  if (c && precision != LSMC_MIXED) {  // a backward pass: jobs of several sub-tiles
+    const uint32_t ctas = (uint32_t)occupancy(nullptr, precision, basis, plan_ppt(o), o.store) *
+                          (uint32_t)sm_count(nullptr);
+    o.sub = choose_sub_cost(&q, 1, precision, plan_ppt(o), ctas);
+  }
   std::unique_ptr<lsmc_plan> p(new (std::nothrow) lsmc_plan());
   if (!p) return LSMC_ENOMEM;
   p->stream = s;
@@ -1608,7 +1643,10 @@ int backward_in_scratch(void* scratch, size_t scratch_bytes, const void* d_S, co
   int rc = stage_plan(m, c->T, scheme, precision, P, N, basis, c, 0, 0, s, &p);
   if (rc) return rc;
   std::unique_ptr<lsmc_plan> owner(p);
-  if (p->L.total_bytes > scratch_bytes) return LSMC_ENOMEM;
+  // the documented limit: what jobs of one sub-tile would need
+  const size_t tile = (size_t)backward_tile(precision, plan_ppt(p->L.opt));
+  const size_t partial1 = align256((P + tile - 1) / tile * kNSum * sizeof(double));
+  if (p->L.total_bytes - p->L.bytes_partial + partial1 > scratch_bytes) return LSMC_ENOMEM;
   p->run_forward = p->run_greeks = false;
   p->dev = (char*)scratch;  // borrowed: never freed here
   if (d_beta) rc = cuda_status(cudaMemsetAsync(d_beta, 0xFF, sizeof(double) * 6 * N, s));

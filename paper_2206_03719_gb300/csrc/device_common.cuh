@@ -298,6 +298,10 @@ __device__ __forceinline__ uint32_t ld_volatile(const uint32_t* p) {
   return *(const volatile uint32_t*)p;
 }
 
+__device__ __forceinline__ void prefetch_l1(const void* p) {
+  asm volatile("prefetch.global.L1 [%0];" ::"l"(p));
+}
+
 // L2-coherent loads of data other CTAs wrote during this launch
 __device__ __forceinline__ double ld_cg(const double* p) { return __ldcg(p); }
 __device__ __forceinline__ float ld_cg(const float* p) { return __ldcg(p); }

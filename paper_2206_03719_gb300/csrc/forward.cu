@@ -43,8 +43,13 @@ forward_kernel(FwdArgs a) {
     }
     if (CHK_OK(a.chk, &a.contracts[lo], sizeof(FwdContract))) sc = a.contracts[lo];
     else sc = FwdContract{};
+    if (gridDim.y > 1) {  // a CTA per path group (launch_forward_k)
+      sc.group0 += blockIdx.y;
+      sc.n_groups = blockIdx.y < sc.n_groups ? 1u : 0u;
+    }
   }
   __syncthreads();
+  if (sc.n_groups == 0) return;
   if (threadIdx.x < sc.n_groups && threadIdx.x < kMaxGroups &&
       CHK_OK(a.chk, &a.groups[sc.group0 + threadIdx.x], sizeof(FwdGroup)))
     make_group_const<Real>(a.groups[sc.group0 + threadIdx.x], gc[threadIdx.x]);
@@ -540,12 +545,28 @@ __global__ void draws_kernel(uint2 key, uint32_t stream_id,
   out[3 * i + 2] = zX;
 }
 
+// A CTA takes all path groups of its 128 paths, which then share the step's
+// draws, or one group (grid.y), which fills the chip where paths are few.
+// The kernels are bound by instruction issue (double: by the FP64 pipe of each
+// quarter of an SM), so the time is the CTAs of the fullest SM times a step's
+// instructions: `shared` (draws) + `group` a group.  4096 x 32 in double with
+// three groups: 32 CTAs 167 us, 96 CTAs 83.
+template <typename Real> struct FwdCost {
+  static constexpr uint32_t kShared = std::is_same<Real, double>::value ? 5 : std::is_same<Real, df>::value ? 110 : 70;
+  static constexpr uint32_t kGroup = std::is_same<Real, double>::value ? 26 : std::is_same<Real, df>::value ? 230 : 60;
+};
+
 template <typename Real, int SCHEME, bool SEG, int FMT>
 static cudaError_t launch_forward_k(const FwdArgs& a, cudaStream_t s) {
   const cudaError_t e =
       allow_dynamic<forward_kernel<Real, SCHEME, SEG, FMT>>(tab_bytes<Real>());
   if (e != cudaSuccess) return e;
-  forward_kernel<Real, SCHEME, SEG, FMT><<<a.n_blocks, kFwdBlock, tab_bytes<Real>(), s>>>(a);
+  const uint64_t sms = a.sms ? a.sms : 1, g = a.max_groups ? a.max_groups : 1;
+  auto waves = [&](uint64_t ctas) { return (ctas + sms - 1) / sms; };
+  const uint64_t together = waves(a.n_blocks) * (FwdCost<Real>::kShared + g * FwdCost<Real>::kGroup);
+  const uint64_t apart = waves(a.n_blocks * g) * (FwdCost<Real>::kShared + FwdCost<Real>::kGroup);
+  const dim3 grid(a.n_blocks, apart < together ? (unsigned)g : 1u);
+  forward_kernel<Real, SCHEME, SEG, FMT><<<grid, kFwdBlock, tab_bytes<Real>(), s>>>(a);
   return cudaGetLastError();
 }
 

@@ -104,6 +104,8 @@ struct FwdArgs {
   unsigned long long next_job_value;
   uint32_t stream_xor;  // xored into every contract's stream id (pricing paths)
   int32_t store_fmt;    // element type of the E/V rows (kStore*)
+  uint32_t max_groups;  // largest n_groups of a contract
+  uint32_t sms;         // SMs of the device
   // every contract of the launch draws under one key: its Philox round keys
   // (key advanced r times at 2r, 2r + 1); uniform_key = 0 otherwise
   int32_t uniform_key;
@@ -219,6 +221,7 @@ struct BwdArgs {
   unsigned long long timeout_ns;
   uint32_t n_rounds, n_inst;
   uint32_t row0;             // date of E/V row index 0 of the instances' rows
+  uint32_t poll_ns;          // longest back-off of a wait
   int32_t store_fmt;         // element type of the E/V rows (kStore*)
   // Per-request completion (serving): the last instance of a request to
   // finish forms the request's price and Greeks and hands them to the host

@@ -191,6 +191,39 @@ uint32_t choose_sub(const lsmc_request* reqs, size_t n, int precision, int ppt,
   return (uint32_t)std::min<uint64_t>(kMaxSub, std::max<uint64_t>(1, sub));
 }
 
+uint32_t choose_sub_cost(const lsmc_request* reqs, size_t n, int precision, int ppt,
+                         uint32_t workers) {
+  const uint64_t tile0 = (uint64_t)backward_tile(precision, ppt);
+  const double w = std::max<uint32_t>(1, workers);
+  static const uint32_t kCandidates[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, kMaxSub};
+  uint32_t best = 1;
+  double best_cost = HUGE_VAL;
+  for (uint32_t sub : kCandidates) {
+    double first = 0.0, total = 0.0, rounds = 1.0, tiles_max = 1.0;
+    for (size_t i = 0; i < n; ++i) {
+      std::vector<Scenario> sc;
+      if (expand_scenarios(reqs[i], &sc) < 0) continue;
+      const double tiles = (double)((reqs[i].n_paths + tile0 * sub - 1) / (tile0 * sub));
+      const double dates = reqs[i].style == LSMC_EUROPEAN ? 1.0 : (double)reqs[i].n_steps;
+      const double jobs = tiles * (double)(sc.size() * reqs[i].n_strikes);
+      first += jobs;
+      total += jobs * dates;
+      rounds = std::max(rounds, dates);
+      tiles_max = std::max(tiles_max, tiles);
+    }
+    // jobs per CTA and date, between the first date's and the average one's
+    const double x = std::sqrt(first * (total / rounds)) / w;
+    const double busy = x < 1.0 ? 1.2 : x + 0.8 * (std::ceil(x) - x);
+    const double cost = (busy + 0.4) * (sub + 2.0) + 1.5 * std::min(1.0, 1.0 / std::max(x, 1e-9)) +
+                        0.015 * tiles_max;
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = sub;
+    }
+  }
+  return best;
+}
+
 int build_layout(const lsmc_request* reqs, size_t n, const PlanOptions& opt,
                  PlanLayout* L) {
   *L = PlanLayout();

@@ -80,6 +80,22 @@ bool itm_at_spot(const lsmc_request& q, uint32_t k);
 uint32_t choose_sub(const lsmc_request* reqs, size_t n, int precision, int ppt,
                     uint32_t workers, uint32_t jobs_per_worker = 4);
 
+// Sub-tiles per backward job of the double and float-pair passes: the least of
+// a cost per date in units of a sub-tile's time on a CTA (4 us).  A job costs
+// its sub-tiles and 2 more (taking, wait, reduction, arrival: 7.4 us measured
+// against 4.0 a sub-tile); with x jobs per CTA the last wave is partly empty
+// (0.8 of the missing part; 1.2 jobs below one a CTA) and the strikes' jobs are
+// uneven (0.4 of a job); with few jobs per CTA a date's solve is not hidden
+// (1.5), and its CTA adds the regression's tiles (0.015 each).  Fitted to
+// sweeps: 131,072 x 252 x 55 regressions, double: 28.6 ms at 8 sub-tiles, 27.4
+// at 12, 34.0 at 16, 31.7 at the 5 that four jobs per CTA gave; float pairs
+// 26.9, 25.0, 27.7, 30.8; 22 regressions of 50,003 paths 5.2 ms at 1, 3.5 at 2,
+// 3.9 at 4; one of 100,001 paths 1.26 ms at 1, 0.99 at 2.  The order of the
+// sums follows the shape: single precision, whose sums round enough to be
+// seen, keeps choose_sub's.
+uint32_t choose_sub_cost(const lsmc_request* reqs, size_t n, int precision, int ppt,
+                         uint32_t workers);
+
 // Sizes and host tables of one launch; device pointers are bound later.
 struct PlanLayout {
   PlanOptions opt;
