@@ -778,34 +778,52 @@ backward_kernel(BwdArgs a) {
     uint32_t ties = 0;
 
     const unsigned lane_lt = (1u << lane) - 1u;
+    // element p of a row: from the sub-tile's base pointer with a constant
+    // offset (float, pairs: no address arithmetic per element), or by its index
+    // (double, where the base pointers' registers cost more: 40.1 against 37.7
+    // ms of the 131,072 x 252 book)
+    auto at = [](auto* row, auto* base, uint32_t p, int k) {
+      return kFixed ? row + p : base + k * kBT;
+    };
     if constexpr (!kCompact) {
       // single precision: one predicated pass per sub-tile (bound by loads)
-      for (uint32_t sb = 0; sb < sub; ++sb) {
-        const uint32_t sub_base = tile_base + sb * TILE0;
-        if (sub_base >= P) break;  // uniform across the CTA
+      // single precision, one predicated pass per sub-tile, bound by instruction
+      // issue: full sub-tiles run without the path bound, rows by a base
+      // pointer and constant offsets (1,048,576 x 252 book 154 -> 138
+      // instructions a path and date, 80.1 -> 70 ms)
+      auto sub_tile = [&](auto is_full, uint32_t sb, uint32_t sub_base) {
+        constexpr bool kFull = decltype(is_full)::value;
         const uint32_t p_base = sub_base + tid;
+        // rows by a base pointer and constant offsets
+        const size_t pb = p_base;
+        const St* qN = EN + pb;
+        const St* q1 = E1 + pb;
+        const St* w1 = BASIS == kBasisSV2 ? V1 + pb : nullptr;
+        const St* q0 = final_job ? nullptr : E0 + pb;
+        const St* w0 = (BASIS == kBasisSV2 && !final_job) ? V0 + pb : nullptr;
+        Real* zp = Z + pb;
         // every load of the sub-tile is issued before any arithmetic, so each
         // thread has up to 5 * PPT independent loads in flight
         Real zr[PPT];
         St e1r[PPT], v1r[PPT], e0r[PPT], v0r[PPT];
 #pragma unroll
         for (int k = 0; k < PPT; ++k) {
-          const uint32_t p = p_base + k * kBT;
+          const bool in = kFull || p_base + k * kBT < P;
           zr[k] = (Real)0;
           e1r[k] = v1r[k] = e0r[k] = v0r[k] = (St)0;
-          if (p < P) {
+          if (in) {
             if (first) {
-              e1r[k] = CHK_LD(a.chk, &EN[p]);
+              e1r[k] = CHK_LD(a.chk, &qN[k * kBT]);
             } else {
-              zr[k] = CHK_OK(a.chk, Z + p, sizeof(Real)) ? ld_cg(Z + p) : (Real)0;
+              zr[k] = CHK_OK(a.chk, &zp[k * kBT], sizeof(Real)) ? ld_cg(&zp[k * kBT]) : (Real)0;
               if (bok) {
-                e1r[k] = CHK_LD(a.chk, &E1[p]);
-                if (BASIS == kBasisSV2) v1r[k] = CHK_LD(a.chk, &V1[p]);
+                e1r[k] = CHK_LD(a.chk, &q1[k * kBT]);
+                if (BASIS == kBasisSV2) v1r[k] = CHK_LD(a.chk, &w1[k * kBT]);
               }
             }
             if (!final_job) {
-              e0r[k] = CHK_LD(a.chk, &E0[p]);
-              if (BASIS == kBasisSV2) v0r[k] = CHK_LD(a.chk, &V0[p]);
+              e0r[k] = CHK_LD(a.chk, &q0[k * kBT]);
+              if (BASIS == kBasisSV2) v0r[k] = CHK_LD(a.chk, &w0[k * kBT]);
             }
           }
         }
@@ -821,13 +839,12 @@ backward_kernel(BwdArgs a) {
         if (first) {
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
-            const uint32_t p = p_base + k * kBT;
             z[k] = (Real)0;
-            if (p < P) {
+            if (kFull || p_base + k * kBT < P) {
               const Real h = payoff<Real>(type, K, sN * (Real)e1[k]);
               z[k] = fma(h, dNhi, h * dNlo);
               euro += (double)z[k];
-              if (!final_job) CHK_ST(a.chk, &Z[p], z[k]);
+              if (!final_job) CHK_ST(a.chk, &zp[k * kBT], z[k]);
             }
           }
         } else {
@@ -838,9 +855,8 @@ backward_kernel(BwdArgs a) {
             // fitted continuation value (basis centred at the strike and theta)
 #pragma unroll
             for (int k = 0; k < PPT; ++k) {
-              const uint32_t p = p_base + k * kBT;
               const Real S = s1 * e1[k];
-              if (p < P && in_money<Real>(type, K, S)) {
+              if ((kFull || p_base + k * kBT < P) && in_money<Real>(type, K, S)) {
                 const Real h = intrinsic<Real>(type, K, S);
                 const Real x = qfma(S, invK, (Real)-1);
                 Real c = qfma(qfma(b[2], x, b[1]), x, b[0]);
@@ -855,7 +871,7 @@ backward_kernel(BwdArgs a) {
                 if (exercise) {
                   const Real hz = fma(h, d1, h * d1lo);
                   z[k] = hz;
-                  if (!final_job) CHK_ST(a.chk, &Z[p], hz);
+                  if (!final_job) CHK_ST(a.chk, &zp[k * kBT], hz);
                 }
               }
             }
@@ -864,8 +880,7 @@ backward_kernel(BwdArgs a) {
         if (final_job) {
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
-            const uint32_t p = p_base + k * kBT;
-            if (p < P) {
+            if (kFull || p_base + k * kBT < P) {
               const double zv = (double)z[k];
               sy += zv;
               sy2 += zv * zv;
@@ -876,9 +891,8 @@ backward_kernel(BwdArgs a) {
           Real* t = acc.target();
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
-            const uint32_t p = p_base + k * kBT;
             const Real S = s0 * e0[k];
-            if (p < P && in_money<Real>(type, K, S)) {
+            if ((kFull || p_base + k * kBT < P) && in_money<Real>(type, K, S)) {
               accumulate_moments<Real, BASIS, NM>(t, n_itm, S, v0[k], z[k], invK, invTh);
             }
           }
@@ -888,6 +902,12 @@ backward_kernel(BwdArgs a) {
           // with one per two, 77.9 with one per four
           if ((sb & 3u) == 3u) acc.fold();
         }
+      };
+      for (uint32_t sb = 0; sb < sub; ++sb) {
+        const uint32_t sub_base = tile_base + sb * TILE0;
+        if (sub_base >= P) break;  // uniform across the CTA
+        if (P - sub_base >= (uint32_t)TILE0) sub_tile(std::true_type{}, sb, sub_base);
+        else sub_tile(std::false_type{}, sb, sub_base);
       }
       acc.fold();
     } else {
@@ -939,18 +959,17 @@ backward_kernel(BwdArgs a) {
           const uint32_t sub_base = tile_base + sb * TILE0;
           if (sub_base >= P) break;  // uniform across the CTA
           const uint32_t p_base = sub_base + tid;
+          const St* r1 = first ? EN : E1;
+          const St* q1 = r1 + (size_t)p_base;
+          const St* w1 = BASIS == kBasisSV2 ? V1 + (size_t)p_base : nullptr;
           St e1r[PPT], v1r[PPT];
 #pragma unroll
           for (int k = 0; k < PPT; ++k) {
             const uint32_t p = p_base + k * kBT;
             e1r[k] = v1r[k] = (St)0;
             if (p < P) {
-              if (first) {
-                e1r[k] = CHK_LD(a.chk, &EN[p]);
-              } else {
-                e1r[k] = CHK_LD(a.chk, &E1[p]);
-                if (BASIS == kBasisSV2) v1r[k] = CHK_LD(a.chk, &V1[p]);
-              }
+              e1r[k] = CHK_LD(a.chk, at(r1, q1, p, k));
+              if (BASIS == kBasisSV2 && !first) v1r[k] = CHK_LD(a.chk, at(V1, w1, p, k));
             }
           }
           LoadT e1[PPT], v1[PPT];
@@ -1055,6 +1074,9 @@ backward_kernel(BwdArgs a) {
         const uint32_t sub_base = tile_base + sb * TILE0;
         if (sub_base >= P) break;  // uniform across the CTA
         const uint32_t p_base = sub_base + tid;
+        const Real* zp = Z + (size_t)p_base;
+        const St* q0 = final_job ? nullptr : E0 + (size_t)p_base;
+        const St* w0 = (BASIS == kBasisSV2 && !final_job) ? V0 + (size_t)p_base : nullptr;
         Real z[PPT];
         St e0r[PPT], v0r[PPT];
 #pragma unroll
@@ -1063,10 +1085,11 @@ backward_kernel(BwdArgs a) {
           z[k] = (Real)0;
           e0r[k] = v0r[k] = (St)0;
           if (p < P) {
-            z[k] = CHK_OK(a.chk, Z + p, sizeof(Real)) ? ld_cg(Z + p) : (Real)0;
+            const Real* zk = at((const Real*)Z, zp, p, k);
+            z[k] = CHK_OK(a.chk, zk, sizeof(Real)) ? ld_cg(zk) : (Real)0;
             if (!final_job) {
-              e0r[k] = CHK_LD(a.chk, &E0[p]);
-              if (BASIS == kBasisSV2) v0r[k] = CHK_LD(a.chk, &V0[p]);
+              e0r[k] = CHK_LD(a.chk, at(E0, q0, p, k));
+              if (BASIS == kBasisSV2) v0r[k] = CHK_LD(a.chk, at(V0, w0, p, k));
             }
           }
         }
