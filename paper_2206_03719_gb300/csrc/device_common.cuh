@@ -158,6 +158,13 @@ template <> struct TabOf<double> { using type = F64Tables; };
 template <> struct TabOf<df> { using type = DfTables; };
 template <typename Real> using Tab = typename TabOf<Real>::type;
 
+// The tails beyond the tabulated octaves, out of line: one draw in a thousand
+// takes them, and a copy per draw would push the steppers' loops out of the
+// instruction cache.
+static __device__ __noinline__ double quantile_tail_f64(double p) {
+  return norm_quantile_f64(p, 1.0 - p);
+}
+
 // Random inputs of one path step from one Philox block: the uniform U_V,
 // 1 - U_V (exact in both grids), Z_V = Phi^-1(U_V) and Z_X.  The float-pair
 // specialisation is in df_math.cuh.
@@ -213,8 +220,7 @@ template <> struct Draw<double> {
       p.lo = __fmaf_rn(g.hi, tl, __fmaf_rn(g.lo, t, p.lo));
       z = tab->q0[j] + (widen_float(p.hi) + widen_float(p.lo));
     } else {
-      const double p = grid_point(ph, pl & 0xfffff000u);
-      z = norm_quantile_f64(p, 1.0 - p);
+      z = quantile_tail_f64(grid_point(ph, pl & 0xfffff000u));
     }
     return __hiloint2double(__double2hiint(z) ^ (int)(s & 0x80000000u), __double2loint(z));
   }

@@ -172,6 +172,11 @@ __device__ __forceinline__ df normal_quantile_lower_df(df p, const DfTables* t) 
   return quick_two_sum(s.hi, __fadd_rn(s.lo, __fsub_rn(corr, d.lo)));
 }
 
+// The tail beyond the tabulated octaves, out of line as in Draw<double>.
+static __device__ __noinline__ df quantile_tail_df(uint32_t hi, uint32_t l21, const DfTables* t) {
+  return normal_quantile_lower_df(uniform_pair(hi, l21), t);
+}
+
 // The random inputs of one path step from one Philox block, as pairs:
 // u = (m + 1/2) 2^-52 from words (0, 1) (the FP64 grid), 1 - u, and the two
 // normal quantiles of the FP64 grid points of words (0, 1) and (2, 3).
@@ -211,7 +216,7 @@ template <> struct Draw<df> {
       z = two_sum(c0.x, p.hi);
       z = quick_two_sum(z.hi, __fadd_rn(z.lo, __fadd_rn(c0.y, p.lo)));
     } else {
-      z = normal_quantile_lower_df(uniform_pair(ph, pl >> 11), tab);
+      z = quantile_tail_df(ph, pl >> 11, tab);
     }
     return s ? -z : z;
   }

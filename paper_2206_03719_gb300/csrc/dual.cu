@@ -150,7 +150,11 @@ __global__ void __launch_bounds__(kDualBlock) dual_inner_kernel(DualArgs a) {
   __shared__ GroupConst<Real> gc;
   extern __shared__ __align__(16) unsigned char tab_raw[];
   Tab<Real>* tabs = reinterpret_cast<Tab<Real>*>(tab_raw);
-  __shared__ double s_acc[kMaxDualStrikes][kDualBlock];
+  // sums per strike and thread, after the tables (as many rows as strikes: a
+  // fixed 16 would take 16 KB and two of six resident CTAs)
+  static_assert(tab_bytes<Real>() % sizeof(double) == 0, "rows of doubles");
+  double(*s_acc)[kDualBlock] =
+      reinterpret_cast<double(*)[kDualBlock]>(tab_raw + tab_bytes<Real>());
   __shared__ uint32_t s_ties[kDualBlock];
   __shared__ const Real* s_tab[kMaxDualStrikes];
   __shared__ const ScreenConsts* s_scr[kMaxDualStrikes];
@@ -326,12 +330,13 @@ template <typename Real, int SCHEME, int BASIS>
 static cudaError_t launch_dual_t(const DualArgs& a, cudaStream_t s) {
   constexpr size_t dyn = tab_bytes<Real>();
   cudaError_t e = allow_dynamic<dual_outer_kernel<Real, SCHEME>>(dyn);
-  if (e == cudaSuccess) e = allow_dynamic<dual_inner_kernel<Real, SCHEME, BASIS>>(dyn);
+  const size_t sums = (size_t)a.n_strikes * kDualBlock * sizeof(double);
+  if (e == cudaSuccess) e = allow_dynamic<dual_inner_kernel<Real, SCHEME, BASIS>>(dyn + sums);
   if (e == cudaSuccess) e = allow_dynamic<dual_max_kernel<Real, SCHEME, BASIS>>(dyn);
   if (e != cudaSuccess) return e;
   dual_outer_kernel<Real, SCHEME>
       <<<(a.n_outer + kDualBlock - 1) / kDualBlock, kDualBlock, dyn, s>>>(a);
-  dual_inner_kernel<Real, SCHEME, BASIS><<<a.n_outer * a.N, kDualBlock, dyn, s>>>(a);
+  dual_inner_kernel<Real, SCHEME, BASIS><<<a.n_outer * a.N, kDualBlock, dyn + sums, s>>>(a);
   dual_max_kernel<Real, SCHEME, BASIS>
       <<<dim3((a.n_outer + kDualBlock - 1) / kDualBlock, a.n_strikes), kDualBlock, dyn, s>>>(a);
   dual_sum_kernel<<<a.n_strikes, kDualBlock, 0, s>>>(a);
