@@ -65,7 +65,7 @@ enum { LSMC_BASIS_S2 = 0, LSMC_BASIS_SV2 = 1 };
  * estimator in double.
  * DF: paths, regression features, sums and exercise decisions in
  * unevaluated pairs of floats (about 48 significant bits, computed on the
- * FP32 pipes; the normal quantiles, the solve and the estimator in double):
+ * FP32 pipes; the solve and the estimator in double):
  * FP64-grade results at single-precision pipe rates.  Stored values are
  * float pairs, as wide as doubles. */
 enum { LSMC_FP64 = 0, LSMC_MIXED = 1, LSMC_DF = 2 };
@@ -488,8 +488,10 @@ int lsmc_philox(const uint32_t* d_ctr, uint32_t key_lo, uint32_t key_hi,
  * per path and step of Sec. 2.2.1: d_path, d_step (device, n uint32 each);
  * d_out (device) is n x 3 (U_V, Z_V, Z_X) as double (LSMC_FP64: 52-bit
  * grid), float (LSMC_MIXED: 23-bit grid) or float pairs (LSMC_DF: the FP64
- * values split).  Asynchronous on cuda_stream; LSMC_EINVAL for NULL arrays
- * with n > 0 or an unknown precision, LSMC_ECUDA if the launch fails. */
+ * grid points split, their own quantile).  Phi^-1 in double and float pairs
+ * from tabulated segments, within 6e-16 and 1.3e-14, max(1, |z|) relative.
+ * Asynchronous on cuda_stream; LSMC_EINVAL for NULL arrays with n > 0 or an
+ * unknown precision, LSMC_ECUDA if the launch fails. */
 int lsmc_draws(uint64_t seed, uint32_t stream_id, const uint32_t* d_path,
                const uint32_t* d_step, size_t n, int32_t precision,
                void* d_out, void* cuda_stream);
@@ -506,7 +508,8 @@ int lsmc_exp(const void* d_x, void* d_y, size_t n, int32_t precision, void* cuda
  * of the Heston step from uniforms) on n uniforms: d_u, d_z (device) double
  * (LSMC_FP64) or float (LSMC_MIXED); z = Phi^-1(u) with 1 - u formed in the
  * precision, exact for u on its uniform grid (the points (m + 1/2) 2^-52,
- * (m + 1/2) 2^-23 that lsmc_draws uses).  Double: w = -log(4 u (1 - u)) by
+ * (m + 1/2) 2^-23 that lsmc_draws uses; in double lsmc_draws' z, from
+ * tables, may differ in the last bit).  Double: w = -log(4 u (1 - u)) by
  * a table-driven logarithm and polynomials in w or sqrt(w) (Giles'
  * transformation, own fit), within 6e-16 of Phi^-1(u), max(1, |z|)
  * relative; float: within 1e-6.  Asynchronous on cuda_stream; LSMC_EINVAL for
