@@ -62,18 +62,22 @@ STEP_GROUP = {"qe": {"flops": 26, "functions": 6}, "ft_euler": {"flops": 13, "fu
 #     5 multiply-adds for the continuation value, compare             -> 15
 BWD_FLOPS_ALL = 3
 BWD_FLOPS_ITM = 40 + 15
-# DRAM bytes of one FP64 backward launch on the 131,072-path book, from an
-# ncu capture (dram__bytes_read.sum + dram__bytes_write.sum) of the same
-# kernel at 98,304 paths (3.110958e9 + 0.348644e9 bytes) scaled by the path
-# count (the path store and cash flows grow in proportion).  Valid only for
-# the kernel source and the tile shape it was taken with (sub-tiles per job
-# with LSMC_SUB_ITM_HALF, paths per lane): reported as null once the code of
-# backward.cu changes (code_sha256_16) or the bench runs another shape.
-BWD_TRAFFIC = {"bytes": (3.110957824e9 + 0.348643840e9) * 131072 / 98304,
-               "source_sha256_16": "9312333d9ec49f23",
-               "shape": (32 | 0x8000, 2),
-               "capture": "profiles/backward_kernel_fp64_98304x252.md (traffic capture), "
-                          "scaled by 131072/98304"}
+# An ncu capture of the FP64 backward kernel, 98,304 paths x 252 dates x 55
+# regressions: instructions per (regression, path, date), 32 x
+# smsp__inst_executed over their number (idle lanes count, as their issue
+# slots are spent; 339), and DRAM bytes (dram__bytes_read.sum +
+# dram__bytes_write.sum) scaled to the 131,072-path book (the path store and
+# cash flows grow in proportion).  Instruction issue bounds the kernel: its
+# moment sums are integer multiply-adds and its exercise test mostly runs in
+# single precision, so the double-precision pipe is a quarter busy.  Valid only
+# for the source (null once the code of backward.cu changes, code_sha256_16) and
+# the paths per lane it was taken with; the bytes only for its sub-tiles per job
+# too (the instructions differ by 4% between 8 and 12).
+BWD_CAPTURE = {"inst_per_path_date": 14436149846 * 32 / (98304 * 252 * 55),
+               "bytes": (3.618812672e9 + 0.476762624e9) * 131072 / 98304,
+               "shape": (12, 4),
+               "source_sha256_16": "a34b339966f7448e",
+               "file": "profiles/backward_kernel_fp64_98304x252.md"}
 
 
 def code_sha256_16(path):
@@ -880,28 +884,36 @@ def main():
         gold = json.load(open(GOLDEN))["results"]
         acc = max_rel_err(res, gold)
 
-    fp64_peak = RUN["peaks"].get("fp64_tflops")
     bwd_ms = kms[2] / max(1, launches)
     fwd_ms = kms[1] / max(1, launches)
     itm = info.itm_path_steps
     flops = BWD_FLOPS_ALL * info.lsmc_path_steps + BWD_FLOPS_ITM * itm
-    achieved = flops / (bwd_ms / 1e3) / 1e12
     fp64 = wl.precision == "fp64"
-    traffic = None
+    # issue rate: one warp instruction per scheduler and clock, measured as the
+    # single-precision fused multiply-add rate (two operations each)
+    fp32_peak = RUN["peaks"].get("fp32_tflops")
+    issue_peak = fp32_peak / 2 if fp32_peak else None
     src = os.path.join(_ROOT, "paper_2206_03719_gb300", "csrc", "backward.cu")
-    if fp64 and wl.n_paths == workloads.PAPER_FP64.n_paths and os.path.exists(src):
-        if (code_sha256_16(src) == BWD_TRAFFIC["source_sha256_16"] and
-                (tuned_sub, tuned_ppt) == BWD_TRAFFIC["shape"]):
-            traffic = BWD_TRAFFIC["bytes"]
+    issued = traffic = None
+    if (fp64 and os.path.exists(src) and tuned_ppt == BWD_CAPTURE["shape"][1] and
+            code_sha256_16(src) == BWD_CAPTURE["source_sha256_16"]):
+        issued = BWD_CAPTURE["inst_per_path_date"] * info.lsmc_path_steps / (bwd_ms / 1e3) / 1e12
+        if (wl.n_paths == workloads.PAPER_FP64.n_paths and
+                (tuned_sub, tuned_ppt) == BWD_CAPTURE["shape"]):
+            traffic = BWD_CAPTURE["bytes"]
     roofline = {
         "kernel": "backward_kernel (Longstaff-Schwartz moments, solve, exercise)",
-        "bound": "alu", "achieved": achieved,
-        "peak": fp64_peak if fp64 else None, "unit": "TFLOP/s",
-        "frac": achieved / fp64_peak if fp64 and fp64_peak else None,
-        "peak_source": "measured: FP64 fused multiply-add probe (lsmc_measure_peaks, "
-                       "%.1f ms on every SM) in this run" % RUN["peaks"].get("fp64_ms", 0.0),
+        "bound": "issue", "achieved": issued, "peak": issue_peak, "unit": "Tinst/s",
+        "frac": issued / issue_peak if issued and issue_peak else None,
+        "peak_source": "measured: FP32 fused multiply-add probe (lsmc_measure_peaks) in this "
+                       "run, one instruction per two operations",
+        "instructions_source": BWD_CAPTURE["file"] if issued else None,
+        # the method's double operations per second; most of them run as integer
+        # or single-precision instructions, so this may exceed the FP64 rate
+        "algorithmic_tflops": flops / (bwd_ms / 1e3) / 1e12,
+        "fp64_peak_tflops": RUN["peaks"].get("fp64_tflops"),
         "traffic": traffic,
-        "traffic_source": BWD_TRAFFIC["capture"] if traffic else None,
+        "traffic_source": BWD_CAPTURE["file"] + ", scaled by 131072/98304" if traffic else None,
         # the path store read once (E and v rows of every path group and date)
         "path_store_bytes": wl.n_paths * wl.n_steps * 2 * 8 *
                             (1 + 2 * ("vega" in wl.greeks) + 2 * ("theta" in wl.greeks)),
