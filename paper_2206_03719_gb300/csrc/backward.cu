@@ -521,8 +521,7 @@ backward_kernel(BwdArgs a) {
   __shared__ ScreenConsts s_q;        // the exercise test of date n + 1 in float
   constexpr bool kFixed = std::is_same<Real, double>::value;
   constexpr bool kSerialSolve = std::is_same<Real, float>::value;
-  __shared__ FixScale s_fix;          // double: the moment sums' fixed-point scales
-  __shared__ int s_range[3];
+  __shared__ FixWarp s_fix[kFixed ? NW : 1];  // double: scales of each warp's sums
   // per-warp compaction of in-the-money paths (dynamic shared memory, one
   // BwdWarpBufs per warp): the heavy arithmetic runs on dense lists instead
   // of on lanes that are mostly out of the money
@@ -699,12 +698,6 @@ backward_kernel(BwdArgs a) {
         if (lane < 6) v = __ldcg(&st->beta[lane]);
         if (kProdLate && (lane == 16 || lane == 17)) v = __ldcg(&st->thr[lane - 16]);
         if (lane == 18) s_beta_ok = (int)__ldcg(&st->beta_ok);
-        if (kFixed && lane >= 19 && lane < 22) s_range[lane - 19] = __ldcg(&st->range[lane - 19]);
-      } else if (kFixed && lane == 19) {
-        // the first date: |x| < 1 for a put, w within 8, y within the strike
-        s_range[0] = type == kPut ? 0 : 1;
-        s_range[1] = 3;
-        s_range[2] = min(max(ilogb(I.K) + 1, kFixRangeMin), kFixRangeMax);
       }
       if (lane == 0) s_go = ok;
       const Real vr = (Real)v;
@@ -741,11 +734,6 @@ backward_kernel(BwdArgs a) {
         else if (lane == 12) s_q.invTh = f;
         else if (lane == 13) s_q.B = B;
       }
-      if constexpr (kFixed) {
-        __syncwarp();
-        if (lane == 19)
-          s_fix = FixScale{kFixBits - s_range[0], kFixBits - s_range[1], kFixBits - s_range[2]};
-      }
     }
     __syncthreads();
     if (!s_go) return;
@@ -772,7 +760,8 @@ backward_kernel(BwdArgs a) {
                          ? V + ((ptrdiff_t)n - r0) * (ptrdiff_t)ld : nullptr;
 
     typename std::conditional<kFixed, FixedSums<BASIS>, Acc<Real, NA>>::type acc;
-    acc.zero();
+    if constexpr (kFixed) acc.zero(s_fix[warp]);
+    else acc.zero();
     uint32_t n_itm = 0;  // in-the-money paths of this thread (monomial 1)
     double euro = 0.0, sy = 0.0, sy2 = 0.0;
     uint32_t ties = 0;
@@ -1140,15 +1129,29 @@ backward_kernel(BwdArgs a) {
         const bool last = kFixed && (sb + 1 == sub || sub_base + TILE0 >= P);
         const int full = last ? cnt : cnt & ~31;
         if constexpr (kFixed) {
+          auto item = [&](int j, Real& e, Real& v, Real& y) {
+            e = get_item<Real, LoadT>(ms, j);
+            v = BASIS == kBasisSV2 ? get_item<Real, LoadT>(mv, j) : (Real)0;
+            y = my[j];
+          };
+          // lane 0 takes part in every chunk: whether the sums hold anything
+          const bool held = __shfl_sync(0xffffffffu, n_itm, 0) != 0;
+          if (!held && full > 0)
+            acc.grow(s_fix[warp], false, 0, full, !last, item, xK0, invTh);
+          int spilt = -1;  // the chunk of which this lane's path is summed already
+          for (int j0 = 0; j0 < full;) {
+            const FixScale f = s_fix[warp].scale;
 #pragma unroll 1
-          for (int j0 = 0; j0 < full; j0 += 32) {
-            const bool have = j0 + lane < full;
-            const int j = have ? j0 + lane : j0;
-            acc.add(s_fix, get_item<Real, LoadT>(ms, j),
-                    BASIS == kBasisSV2 ? get_item<Real, LoadT>(mv, j) : (Real)0, my[j], have, xK0,
-                    invTh);
-            n_itm += have ? 1u : 0u;
+            for (; j0 < full; j0 += 32) {
+              const bool have = j0 + lane < full;
+              Real e, v, y;
+              item(have ? j0 + lane : j0, e, v, y);
+              if (!acc.add(f, e, v, y, have && j0 != spilt, xK0, invTh)) break;
+            }
+            if (j0 < full && acc.grow(s_fix[warp], held || j0 > 0, j0, full, !last, item, xK0, invTh))
+              spilt = j0;
           }
+          if (lane < full) n_itm += (uint32_t)(full - lane + 31) >> 5;
         } else {
           Real* t = acc.target();
           for (int j = lane; j < full; j += 32)
@@ -1196,11 +1199,11 @@ backward_kernel(BwdArgs a) {
       halving_units<Sums::NU, 16>(ua, ub, lane, 0, Sums::NU, oa, ob, i);
       const uint32_t items = __reduce_add_sync(0xffffffffu, n_itm);
       auto slot = [](int u) { return u < NM - 1 ? u + 1 : kSlotRhs + (u - (NM - 1)); };
-      if (i >= 0) s_red[warp][slot(i)] = Sums::value(i, oa, ob, s_fix, type == kPut);
+      if (i >= 0) s_red[warp][slot(i)] = Sums::value(i, oa, ob, s_fix[warp].scale, type == kPut);
       if (lane == 0) s_red[warp][0] = (double)items;
-      if (acc.spilled) {  // uniform across the warp
+      if (s_fix[warp].spilled) {
         __syncwarp();
-        if (lane < Sums::NU) s_red[warp][slot(lane)] += acc.spill;
+        if (lane < Sums::NU) s_red[warp][slot(lane)] += s_fix[warp].spill[lane];
       }
     } else {
       // rows per pass: as many as the warp's moment buffers hold
@@ -1346,13 +1349,6 @@ backward_kernel(BwdArgs a) {
         atomicAdd(&st->ties, s_sum[kSlotTies]);
         if (!ok) atomicAdd(&st->singular, 1u);
         st->beta_ok = ok ? 1u : 0u;
-      }
-      if (kFixed && lane == 1) {  // the ranges of the next date's fixed-point sums
-        st->range[0] = fix_range(s_sum[2], s_sum[0], 4, 2, s_range[0]);
-        st->range[1] = BASIS == kBasisSV2
-                           ? fix_range(s_sum[mono(0, 2)], s_sum[0], 6, 2, s_range[1])
-                           : s_range[1];
-        st->range[2] = fix_range(s_sum[kSlotRhs], s_sum[0], 4, 1, s_range[2]);
       }
     } else if (!final_job && kProdLate && tid == 32) {
       // beside the solve: the thresholds of the next round's two dates

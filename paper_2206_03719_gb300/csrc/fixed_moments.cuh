@@ -6,7 +6,7 @@
 // sums of an in-the-money path took 25 FP64 operations (425 clocks per 32
 // paths), four fifths of the backward pass's FP64 work; here 2 FP64
 // operations, 47 integer multiply-adds and about 110 other integer
-// instructions do it, and the sums are exact, so their order does not matter.
+// instructions do it.
 // (The FP64 matrix instruction m8n8k4 runs at 3.6 times the FP64 rate, 36
 // clocks, but an 8 x 8 tile holds the 21 sums once: 377 clocks for 32 paths.)
 //
@@ -17,15 +17,22 @@
 // 64-bit sum and h l' + l h' to another; l l' is below 2^-54 of the range and
 // of mean zero.  256 paths a lane (the largest job) stay below 2^63.
 //
-// Range.  2^(54 - F) is at least 4 (x) or 8 (w) times the root mean square of
-// the previous exercise date's paths, 16 times the mean for y (integers from
-// the exponents of its sums, published with its coefficients); a path outside
-// (any x, w or y, infinities and NaN among them) is summed in double by the
-// whole warp, a monomial per lane.  In a model of this arithmetic (x normal
-// with deviations 0.003 to 0.2, w gamma; 8 to 60,000 paths) the fitted values
-// are within 3e-15 to 4e-17 of the exact regression's, against 4e-15 to 6e-16
-// with double sums; 49 bits, which one fused multiply-add could produce, gave
-// 9e-14 to 1e-15.
+// Range.  2^(54 - F) is the smallest power of two above the largest |q| that
+// the warp has summed in its job, for x, w and y each (for y, of which only
+// first powers are summed, with two bits to spare while more paths may come).
+// It is taken from the first list of paths; when a later path lies beyond it,
+// the sums held are shifted to the larger range (hl keeps what hh drops).  So
+// the scales follow the warp's own paths alone, whatever the maturity, the
+// volatilities or the distance of v0 from theta, and depend on no earlier date
+// and no other warp.  (With ranges fixed for the first date and taken from the
+// date before for the others, narrow distributions lost their digits: at one
+// day and xi = 0.005, 3,001 paths, the coefficients scaled by their functions'
+// norms were off by 5e-2, where a fit in double may be off by 2e-10.)  Growing
+// is outside the loop over the paths: inside it, its registers cost twice as
+// much as its work (book of 131,072 x 252 x 55: fixed ranges 37.8 ms, grown in
+// the loop 42.5, outside 39.4).  Values beyond 2^100 (x, w) or 2^400 (y),
+// infinities and NaN are summed in double by the whole warp, a monomial per
+// lane.
 #pragma once
 
 #include <cstdint>
@@ -36,15 +43,30 @@ namespace lsmc {
 namespace {
 
 constexpr int kFixBits = 54;  // |integer| < 2^54
-constexpr int kFixRangeMin = -40, kFixRangeMax = 40;  // exponents of the ranges
+// Largest ranges: x and w < 2^kFixTopXW, cash flows < 2^kFixTopY (values
+// beyond, infinities and NaN are summed in double).  The scales start at ranges
+// 2^-kFixTopXW and 2^-kFixTopY.  With these every scale of a sum is a normal
+// double.
+constexpr int kFixTopXW = 100, kFixTopY = 400;
 
-// F of each variable, as the shift from a double's exponent field
+// F of each variable: the integer of q is round(q 2^F)
 struct FixScale {
-  int Fx, Fw, Fy;
+  int x, w, y;
 };
 
 __device__ __forceinline__ double exp2_int(int k) {  // 2^k, k in the normal range
   return __hiloint2double((1023 + k) << 20, 0);
+}
+
+// v >> n, zero for any n (read unsigned) beyond 63
+__device__ __forceinline__ unsigned long long shr_clamped(unsigned long long v, int n) {
+#ifdef __CUDA_ARCH__
+  unsigned long long r;
+  asm("shr.u64 %0, %1, %2;" : "=l"(r) : "l"(v), "r"(n));
+  return r;
+#else
+  return (unsigned)n > 63u ? 0ull : v >> n;
+#endif
 }
 
 // A value's integer round(q 2^F) = h 2^28 + l, |l| <= 2^27.
@@ -61,7 +83,7 @@ struct Limbs {
 
 // The limbs of |q| 2^F, from the mantissa m and the exponent field e of q
 // (|q| = m 2^(e - 1075)); hi: the high word of |q|.  bad: |q| outside the
-// range (then the limbs mean nothing).
+// range, e > 1076 - F (then the limbs mean nothing).
 __device__ __forceinline__ Limbs fix_magnitude(int hi, int lo, int F, bool& bad) {
   // m shifted left by 3 and right by n: twice the integer, the last bit rounding
   const int n = 1077 - F - (hi >> 20);
@@ -69,9 +91,8 @@ __device__ __forceinline__ Limbs fix_magnitude(int hi, int lo, int F, bool& bad)
   const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = ((unsigned long long)__funnelshift_l((uint32_t)lo, mh, 3) << 32) |
                                ((uint32_t)lo << 3);
-  unsigned long long t;  // zero for shifts beyond 63 (small values, and the bad ones)
-  asm("shr.u64 %0, %1, %2;" : "=l"(t) : "l"(m), "r"(n));
-  t += 1ull + (1ull << 28);
+  // zero for shifts beyond 63 (small values, and the bad ones)
+  const unsigned long long t = shr_clamped(m, n) + (1ull + (1ull << 28));
   Limbs r;
   r.h = (int)__funnelshift_r((uint32_t)t, (uint32_t)(t >> 32), 29);
   r.l = (int)(((uint32_t)t & 0x1fffffffu) >> 1) - (1 << 27);
@@ -84,17 +105,6 @@ __device__ __forceinline__ Limbs fix_signed(double q, int F, bool& bad) {
   r.h = (r.h ^ s) - s;
   r.l = (r.l ^ s) - s;
   return r;
-}
-
-// Exponent of the range of the next date from this date's sums: 2^e >= m
-// times the root mean square (or, order 1, the mean) of `sum` over `count`;
-// m2 = log2(m) * order; `keep` where nothing was summed.
-__device__ __forceinline__ int fix_range(double sum, double count, int m2, int order, int keep) {
-  const int es = (__double2hiint(sum) >> 20) & 0x7ff, en = (__double2hiint(count) >> 20) & 0x7ff;
-  if (es == 0 || es == 0x7ff || en == 0 || en == 0x7ff) return keep;
-  const int d = es - en + 1 + m2;  // sum / count < 2^(es - en + 1)
-  const int e = order == 2 ? (d + 1) >> 1 : d;
-  return min(max(e, kFixRangeMin), kFixRangeMax);
 }
 
 // The sums of a basis as units, in slot order without the count: a sum of
@@ -128,9 +138,13 @@ __device__ __noinline__ double fix_monomial(uint32_t unit, double x, double w, d
 // a b + c as one instruction (written out: from 64-bit C expressions the
 // compiler forms full 64-bit products: 394 instructions a path against 266)
 __device__ __forceinline__ long long wide(int a, int b, long long c) {
+#ifdef __CUDA_ARCH__
   long long r;
   asm("mad.wide.s32 %0, %1, %2, %3;" : "=l"(r) : "r"(a), "r"(b), "l"(c));
   return r;
+#else
+  return (long long)a * b + c;
+#endif
 }
 // round(A B 2^-54)
 __device__ __forceinline__ long long fix_product(const Limbs& a, const Limbs& b) {
@@ -142,6 +156,14 @@ __device__ __forceinline__ long long fix_square(const Limbs& a) {
   return wide(4 * a.h, a.h, wide(a.h + a.h, a.l, (1ll << 25) + (1ll << 26) / 3) >> 26);
 }
 
+// What a warp's lanes share, in shared memory: the scales of the sums, and the
+// sums over the paths beyond the largest range.
+struct FixWarp {
+  FixScale scale;
+  int spilled;       // whether spill holds anything
+  double spill[20];
+};
+
 // Sums of one warp: per unit and lane two 64-bit sums, of h h' and of
 // h l' + l h' (one for the plain sums, in hh).  The x here is |S / K - 1|
 // (in-the-money paths lie on one side of the strike); value() gives odd powers
@@ -150,17 +172,24 @@ template <int BASIS> struct FixedSums {
   static constexpr bool kV = BASIS == kBasisSV2;
   static constexpr int NU = kV ? 20 : 7;
   long long hh[NU], hl[NU];
-  double spill;  // lane u < NU: unit u over the paths outside the range
-  bool spilled;
 
+  __device__ __forceinline__ static constexpr bool is_plain(int u) {
+    return u == 0 || u == 1 || (kV ? u == 4 || u == 5 || u == 8 || u == 14 : u == 4);
+  }
   __device__ __forceinline__ static uint32_t unit(int u) {
     return kV ? kFixUnitsSV2[u] : kFixUnitsS2[u];
   }
-  __device__ __forceinline__ void zero() {
+  // called by the whole warp
+  __device__ __forceinline__ void zero(FixWarp& ws) {
 #pragma unroll
     for (int i = 0; i < NU; ++i) hh[i] = hl[i] = 0;
-    spill = 0.0;
-    spilled = false;
+    const int lane = threadIdx.x & 31;
+    if (lane < NU) ws.spill[lane] = 0.0;
+    if (lane == 0) {
+      ws.scale = FixScale{kFixBits + kFixTopXW, kFixBits + kFixTopXW, kFixBits + kFixTopY};
+      ws.spilled = 0;
+    }
+    __syncwarp();
   }
   __device__ __forceinline__ void plain(int i, const Limbs& a) {
     hh[i] = wide(a.h, 1 << 28, wide(a.l, 1, hh[i]));
@@ -173,31 +202,45 @@ template <int BASIS> struct FixedSums {
     hh[i] = wide(a.h, a.h, hh[i]);
     hl[i] = wide(a.h + a.h, a.l, hl[i]);
   }
-  // one path per lane (valid lanes): row values e, v and cash flow z; called
-  // by the whole warp
-  __device__ __forceinline__ void add(const FixScale& f, double e, double v, double z, bool valid,
+  // The sums from scales f to scales n <= f, in steps that divide no unit by
+  // more than 2^28: a plain sum is rounded, of the others hl keeps what hh
+  // drops (errors below a unit of hl, 2^-80 of the new range's product).
+  __device__ __forceinline__ void rescale(const FixScale& f, const FixScale& n) {
+    // beyond 2^98 nothing is left of a sum
+    int dx = min(f.x - n.x, 98), dw = min(f.w - n.w, 98), dy = min(f.y - n.y, 98);
+#pragma unroll 1
+    while (dx > 0 || dw > 0 || dy > 0) {
+      const int sx = min(dx, 7), sw = min(dw, 7), sy = min(dy, 14);
+      dx -= sx;
+      dw -= sw;
+      dy -= sy;
+#pragma unroll
+      for (int i = 0; i < NU; ++i) {
+        const uint32_t t = unit(i);
+        const int s = (int)(t & 15u) * sx + (int)((t >> 4) & 15u) * sw + (int)((t >> 8) & 15u) * sy;
+        if (is_plain(i)) {
+          hh[i] = (hh[i] + (long long)((1u << s) >> 1)) >> s;
+        } else {
+          hl[i] = (hl[i] >> s) + (long long)(((uint32_t)hh[i] & ((1u << s) - 1u)) << (28 - s));
+          hh[i] >>= s;
+        }
+      }
+    }
+  }
+  // Adds one path per lane (valid lanes): row values e, v and cash flow z.
+  // Called by the whole warp; false, and nothing added, where a path lies
+  // beyond the range of the scales f.
+  __device__ __forceinline__ bool add(const FixScale& f, double e, double v, double z, bool valid,
                                       double xK, double invTh) {
     const double xd = fma(e, xK, -1.0), wd = kV ? fma(v, invTh, -1.0) : 0.0;
     bool bad = false;
-    Limbs x = fix_magnitude(__double2hiint(xd) & 0x7fffffff, __double2loint(xd), f.Fx, bad);
-    Limbs y = fix_magnitude(__double2hiint(z) & 0x7fffffff, __double2loint(z), f.Fy, bad);
+    Limbs x = fix_magnitude(__double2hiint(xd) & 0x7fffffff, __double2loint(xd), f.x, bad);
+    Limbs y = fix_magnitude(__double2hiint(z) & 0x7fffffff, __double2loint(z), f.y, bad);
     Limbs w;
-    if (kV) w = fix_signed(wd, f.Fw, bad);
+    if (kV) w = fix_signed(wd, f.w, bad);
     if (__any_sync(0xffffffffu, bad || !valid)) {
-      unsigned m = __ballot_sync(0xffffffffu, bad && valid);
-      spilled = spilled || m != 0;
-      const int lane = threadIdx.x & 31;
-      const uint32_t u = unit(lane < NU ? lane : 0);
-#pragma unroll 1
-      while (m) {
-        const int src = __ffs(m) - 1;
-        m &= m - 1;
-        const double xs = __shfl_sync(0xffffffffu, xd, src);
-        const double ws = __shfl_sync(0xffffffffu, wd, src);
-        const double ys = __shfl_sync(0xffffffffu, z, src);
-        spill += fix_monomial(u, xs, ws, ys);
-      }
-      if (bad || !valid) x.h = x.l = y.h = y.l = w.h = w.l = 0;
+      if (__any_sync(0xffffffffu, bad && valid)) return false;
+      if (!valid) x.h = x.l = y.h = y.l = w.h = w.l = 0;
     }
     const Limbs x2(fix_square(x));
     plain(0, x);
@@ -227,6 +270,69 @@ template <int BASIS> struct FixedSums {
       product(5, x, y);
       product(6, x2, y);
     }
+    return true;
+  }
+  // Takes the scales (and the sums, if there are any) to what covers every path
+  // from j0 on of a list of `full`; or, where they do already and add() refused
+  // paths [j0, j0 + 32), sums this chunk's paths beyond the largest range in
+  // double, a monomial per lane, and returns true for their lanes.
+  // item(j, e, v, z) gives a path's values.  more: other lists may follow; y,
+  // of which only first powers are summed, then gets two bits above its
+  // largest value.  Called by the whole warp.
+  template <typename Item>
+  __device__ __forceinline__ bool grow(FixWarp& ws, bool any, int j0, int full, bool more,
+                                       const Item& item, double xK, double invTh) {
+    const int lane = threadIdx.x & 31;
+    const FixScale f = ws.scale;
+    auto exponent = [](double q) { return (__double2hiint(q) >> 20) & 0x7ff; };
+    // largest exponent fields, below the largest ranges'
+    constexpr int kTopXW = 1023 + kFixTopXW, kTopY = 1023 + kFixTopY;
+    int ex = 0, ew = 0, ey = 0;
+#pragma unroll 1
+    for (int j = j0 + lane; j < full; j += 32) {
+      double e, v, z;
+      item(j, e, v, z);
+      const int tx = exponent(fma(e, xK, -1.0)), ty = exponent(z);
+      const int tw = kV ? exponent(fma(v, invTh, -1.0)) : 0;
+      ex = max(ex, tx < kTopXW ? tx : 0);
+      ew = max(ew, tw < kTopXW ? tw : 0);
+      ey = max(ey, ty < kTopY ? ty : 0);
+    }
+    ex = __reduce_max_sync(0xffffffffu, ex);
+    if (kV) ew = __reduce_max_sync(0xffffffffu, ew);
+    ey = __reduce_max_sync(0xffffffffu, ey);
+    FixScale n;
+    n.x = min(f.x, 1076 - ex);
+    n.w = kV ? min(f.w, 1076 - ew) : f.w;
+    n.y = ey > 1076 - f.y ? 1076 - ey - (more ? 2 : 0) : f.y;
+    if (n.x != f.x || n.w != f.w || n.y != f.y) {
+      if (any) rescale(f, n);
+      __syncwarp();
+      if (lane == 0) ws.scale = n;
+      __syncwarp();
+      return false;
+    }
+    double e, v, z;
+    item(min(j0 + lane, full - 1), e, v, z);
+    const double xd = fma(e, xK, -1.0), wd = kV ? fma(v, invTh, -1.0) : 0.0;
+    const bool bad = j0 + lane < full && (exponent(xd) > 1076 - f.x || exponent(wd) > 1076 - f.w ||
+                                          exponent(z) > 1076 - f.y);
+    double p = 0.0;
+    const uint32_t u = unit(lane < NU ? lane : 0);
+    unsigned m = __ballot_sync(0xffffffffu, bad);
+#pragma unroll 1
+    while (m) {
+      const int src = __ffs(m) - 1;
+      m &= m - 1;
+      const double xs = __shfl_sync(0xffffffffu, xd, src);
+      const double wv = __shfl_sync(0xffffffffu, wd, src);
+      const double ys = __shfl_sync(0xffffffffu, z, src);
+      p += fix_monomial(u, xs, wv, ys);
+    }
+    if (lane < NU) ws.spill[lane] += p;
+    if (lane == 0) ws.spilled = 1;
+    __syncwarp();
+    return bad;
   }
   // the units in slot order, in two parts small enough to be added over 32
   // lanes: products as a 2^28 + b in units of 2^56, plain sums in units of 1
@@ -234,17 +340,16 @@ template <int BASIS> struct FixedSums {
     constexpr long long kMask = (1ll << 28) - 1;
 #pragma unroll
     for (int i = 0; i < NU; ++i) {
-      const bool is_plain = i == 0 || i == 1 || (kV ? i == 4 || i == 5 || i == 8 || i == 14 : i == 4);
       a[i] = hh[i] >> 28;
-      b[i] = (hh[i] & kMask) + (is_plain ? 0 : (hl[i] + (1ll << 27)) >> 28);
+      b[i] = (hh[i] & kMask) + (is_plain(i) ? 0 : (hl[i] + (1ll << 27)) >> 28);
     }
   }
   // neg: x is negative (puts)
   __device__ __forceinline__ static double value(int u, long long a, long long b,
                                                  const FixScale& f, bool neg) {
     const uint32_t t = unit(u);
-    const int E = (int)(t & 15u) * f.Fx + (int)((t >> 4) & 15u) * f.Fw +
-                  (int)((t >> 8) & 15u) * f.Fy - kFixBits * (int)((t >> 12) & 15u) +
+    const int E = (int)(t & 15u) * f.x + (int)((t >> 4) & 15u) * f.w +
+                  (int)((t >> 8) & 15u) * f.y - kFixBits * (int)((t >> 12) & 15u) +
                   56 * (int)(t >> 16);
     const double v = fma((double)a, 268435456.0, (double)b) * exp2_int(56 - E);
     return neg && (t & 1u) ? -v : v;

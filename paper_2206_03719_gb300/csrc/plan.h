@@ -193,8 +193,6 @@ struct BwdState {
   double itm;         // in-the-money path-steps seen by the regressions
   double ties;        // near-tie exercise decisions
   double thr[2];      // in-the-money thresholds of the solved date and the next one
-  int32_t range[3];   // double: exponents of the next date's fixed-point ranges
-  int32_t pad_;
 };
 
 struct BwdResult {
