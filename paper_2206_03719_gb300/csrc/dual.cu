@@ -331,7 +331,8 @@ static cudaError_t launch_dual_t(const DualArgs& a, cudaStream_t s) {
   constexpr size_t dyn = tab_bytes<Real>();
   cudaError_t e = allow_dynamic<dual_outer_kernel<Real, SCHEME>>(dyn);
   const size_t sums = (size_t)a.n_strikes * kDualBlock * sizeof(double);
-  if (e == cudaSuccess) e = allow_dynamic<dual_inner_kernel<Real, SCHEME, BASIS>>(dyn + sums);
+  constexpr size_t most = dyn + (size_t)kMaxDualStrikes * kDualBlock * sizeof(double);
+  if (e == cudaSuccess) e = allow_dynamic<dual_inner_kernel<Real, SCHEME, BASIS>>(most);
   if (e == cudaSuccess) e = allow_dynamic<dual_max_kernel<Real, SCHEME, BASIS>>(dyn);
   if (e != cudaSuccess) return e;
   dual_outer_kernel<Real, SCHEME>

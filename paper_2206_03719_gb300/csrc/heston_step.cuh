@@ -30,6 +30,9 @@ template <typename Real> __device__ __forceinline__ void load_tables(Tab<Real>* 
   }
 }
 // The kernels' shared memory above 48 KB (static and dynamic) needs an opt-in.
+// It holds for the kernel in the whole process, so `bytes` is the largest size
+// any launch of the kernel takes: with a size per launch, a thread could lower
+// it between another thread's opt-in and launch.
 template <auto Kernel> static cudaError_t allow_dynamic(size_t bytes) {
   if (bytes == 0) return cudaSuccess;
   return cudaFuncSetAttribute(Kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
