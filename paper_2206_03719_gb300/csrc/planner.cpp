@@ -196,16 +196,22 @@ uint32_t choose_sub_cost(const lsmc_request* reqs, size_t n, int precision, int 
   const uint64_t tile0 = (uint64_t)backward_tile(precision, ppt);
   const double w = std::max<uint32_t>(1, workers);
   static const uint32_t kCandidates[] = {1, 2, 3, 4, 5, 6, 8, 10, 12, 16, 20, 24, 32, 48, kMaxSub};
+  // the regressions and dates of every request, once for all candidates
+  std::vector<double> regressions(n, 0.0);
+  for (size_t i = 0; i < n; ++i) {
+    std::vector<Scenario> sc;
+    if (expand_scenarios(reqs[i], &sc) >= 0)
+      regressions[i] = (double)(sc.size() * reqs[i].n_strikes);
+  }
   uint32_t best = 1;
   double best_cost = HUGE_VAL;
   for (uint32_t sub : kCandidates) {
     double first = 0.0, total = 0.0, rounds = 1.0, tiles_max = 1.0;
     for (size_t i = 0; i < n; ++i) {
-      std::vector<Scenario> sc;
-      if (expand_scenarios(reqs[i], &sc) < 0) continue;
+      if (regressions[i] == 0.0) continue;
       const double tiles = (double)((reqs[i].n_paths + tile0 * sub - 1) / (tile0 * sub));
       const double dates = reqs[i].style == LSMC_EUROPEAN ? 1.0 : (double)reqs[i].n_steps;
-      const double jobs = tiles * (double)(sc.size() * reqs[i].n_strikes);
+      const double jobs = tiles * regressions[i];
       first += jobs;
       total += jobs * dates;
       rounds = std::max(rounds, dates);
