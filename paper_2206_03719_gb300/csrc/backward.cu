@@ -533,18 +533,20 @@ backward_kernel(BwdArgs a) {
   // single precision and float pairs reduce through float pairs; double
   // precision through doubles
   constexpr bool kSingle = !std::is_same<Real, double>::value;
-  // compaction pays where the in-the-money arithmetic is heavy (double and
-  // float pairs); plain floats are bound by loads and stay uncompacted
+  // Compaction pays where the in-the-money arithmetic is heavy (double and
+  // float pairs).  Plain floats stay uncompacted: the lists' own instructions
+  // (ballots, stores, carrying remainders) outweigh what idle lanes cost them
+  // (1,048,576 x 252 book: 91.5 ms through the lists, 84.0 predicated, both
+  // measured with 256 x 2 CTAs before the predicated pass went to 70).
+  // Compacted, the in-the-money test needs no product (a threshold on the
+  // stored value): the buffers hold the stored value and S = s e is formed on
+  // the dense lists, where no lane idles.
   constexpr bool kCompact = !std::is_same<Real, float>::value;
-  // double and float pairs: the in-the-money test needs no product (a
-  // threshold on the stored value), so the compaction buffers hold the
-  // stored value and S = s e is formed on the dense lists, where no lane idles
-  constexpr bool kProdLate = kCompact;
   // Job decoding by one thread (kTaker, in another warp than the arrival).  A
   // job number is taken when the CTA arrives with its previous job (only once
   // the CTA can start it).  Job numbers only
   // grow, so the round is found from the last one's; the instance by a binary
-  // search over every s_step-th entry of cum_tiles in shared memory (dependent
+  // search over every cum_step-th entry of cum_tiles in shared memory (dependent
   // global loads here were on the path of every job).  An error recorded by
   // another CTA is seen in the wait for the previous date.
   const uint32_t cum_step = (a.n_inst + kCumTab - 1) / kCumTab;
@@ -662,7 +664,7 @@ backward_kernel(BwdArgs a) {
         case 12: v = I.inv_theta; break;
         case 14: case 15: v = CHK_LD(a.chk, &dtab[N]); break;
         case 17:  // later rounds: formed beside the previous date's solve
-          if (kProdLate && first && !final_job)
+          if (kCompact && first && !final_job)
             v = row_threshold<Real>(type, CHK_LD(a.chk, &stab[n]), I.K);
           break;
         default: break;
@@ -696,13 +698,13 @@ backward_kernel(BwdArgs a) {
       ok = __shfl_sync(0xffffffffu, ok, 0);
       if (!first && ok) {
         if (lane < 6) v = __ldcg(&st->beta[lane]);
-        if (kProdLate && (lane == 16 || lane == 17)) v = __ldcg(&st->thr[lane - 16]);
+        if (kCompact && (lane == 16 || lane == 17)) v = __ldcg(&st->thr[lane - 16]);
         if (lane == 18) s_beta_ok = (int)__ldcg(&st->beta_ok);
       }
       if (lane == 0) s_go = ok;
       const Real vr = (Real)v;
       if (lane < 16) s_c[lane] = vr;
-      if (kProdLate && (lane == 16 || lane == 17)) {
+      if (kCompact && (lane == 16 || lane == 17)) {
         // double: S = RN(s e) is in the money exactly where e passes the
         // date's threshold T (integer comparison of the bits; a float e of a
         // 16-bit store against T rounded up or down).  Float pairs: S = s e <
@@ -749,7 +751,7 @@ backward_kernel(BwdArgs a) {
     const long long thr1 = std::is_same<Real, double>::value ? s_thr[0] : 0;
     const long long thr0 = std::is_same<Real, double>::value ? s_thr[1] : 0;
     // the moment items hold e (double) or S: x = e (s0 / K) - 1 or S / K - 1
-    const Real xK0 = kProdLate ? s0 * invK : invK;
+    const Real xK0 = kCompact ? s0 * invK : invK;
     // row of date d at index d - a.row0 (rows of dates 1..N, or one segment)
     const ptrdiff_t r0 = (ptrdiff_t)a.row0;
     const St* EN = E + ((ptrdiff_t)N - r0) * (ptrdiff_t)ld;
@@ -775,8 +777,7 @@ backward_kernel(BwdArgs a) {
       return kFixed ? row + p : base + k * kBT;
     };
     if constexpr (!kCompact) {
-      // single precision: one predicated pass per sub-tile (bound by loads)
-      // single precision, one predicated pass per sub-tile, bound by instruction
+      // single precision: one predicated pass per sub-tile, bound by instruction
       // issue: full sub-tiles run without the path bound, rows by a base
       // pointer and constant offsets (1,048,576 x 252 book 154 -> 138
       // instructions a path and date, 80.1 -> 70 ms)
@@ -918,7 +919,7 @@ backward_kernel(BwdArgs a) {
           const uint32_t code = wb.xo[j];
           const int pre = (int)(code >> 30);
           const uint32_t p = tile_base + (code & 0x3fffffffu);
-          const Real S = kProdLate ? rmul(s1, get_item<Real, LoadT>(wb.xe, j)) : wb.xe[j];
+          const Real S = rmul(s1, get_item<Real, LoadT>(wb.xe, j));
           const Real h = intrinsic<Real>(type, K, S);
           const Real hd = qmul(h, d1);
           bool exercise = pre == 1;
@@ -996,8 +997,7 @@ backward_kernel(BwdArgs a) {
             const unsigned m = __ballot_sync(0xffffffffu, itm);
             if (itm) {
               const int pos = cnt + __popc(m & lane_lt);
-              if constexpr (kProdLate) put_item<Real, LoadT>(cs, pos, e1[k]);
-              else cs[pos] = s1 * e1[k];
+              put_item<Real, LoadT>(cs, pos, e1[k]);
               if (BASIS == kBasisSV2) put_item<Real, LoadT>(cv, pos, v1[k]);
               co[pos] = (unsigned short)(k * 32 + lane);
             }
@@ -1116,8 +1116,7 @@ backward_kernel(BwdArgs a) {
           const unsigned m = __ballot_sync(0xffffffffu, itm);
           if (itm) {
             const int pos = cnt + __popc(m & lane_lt);
-            if constexpr (kProdLate) put_item<Real, LoadT>(ms, pos, e0[k]);
-            else ms[pos] = s0 * e0[k];
+            put_item<Real, LoadT>(ms, pos, e0[k]);
             if (BASIS == kBasisSV2) put_item<Real, LoadT>(mv, pos, v0[k]);
             my[pos] = z[k];
           }
@@ -1350,7 +1349,7 @@ backward_kernel(BwdArgs a) {
         if (!ok) atomicAdd(&st->singular, 1u);
         st->beta_ok = ok ? 1u : 0u;
       }
-    } else if (!final_job && kProdLate && tid == 32) {
+    } else if (!final_job && kCompact && tid == 32) {
       // beside the solve: the thresholds of the next round's two dates
       st->thr[0] = s_thrd[1];
       if (n > 1) st->thr[1] = row_threshold<Real>(type, CHK_LD(a.chk, &stab[n - 1]), I.K);

@@ -46,13 +46,6 @@ __device__ __forceinline__ uint4 philox4x32_10_rk(uint4 c, const uint32_t (&rk)[
   return c;
 }
 
-// (m + 1/2) 2^-52, m = top 52 bits of (hi:lo): exact, in (0, 1).
-__device__ __forceinline__ double uniform52(uint32_t hi, uint32_t lo) {
-  const unsigned long long m =
-      ((unsigned long long)hi << 20) | (unsigned long long)(lo >> 12);
-  return __fma_rn(__ull2double_rn(m), 0x1p-52, 0x1p-53);
-}
-
 // (m + 1/2) 2^-23, m = top 23 bits of w: exact, in (0, 1).
 __device__ __forceinline__ float uniform23(uint32_t w) {
   return __fmaf_rn(__uint2float_rn(w >> 9), 0x1p-23f, 0x1p-24f);
@@ -170,8 +163,7 @@ static __device__ __noinline__ double quantile_tail_f64(double p) {
 // specialisation is in df_math.cuh.
 template <typename Real> struct Draw;
 template <> struct Draw<double> {
-  // (m + 1/2) 2^-52, m the top 52 bits of (hi:lo), exact as in uniform52, by
-  // one FP64 subtraction: the integer-to-double conversion runs on the FP64
+  // (m + 1/2) 2^-52, m the top 52 bits of (hi:lo), exact, by one FP64 subtraction: the integer-to-double conversion runs on the FP64
   // pipe as well (15 clocks a warp) and needs two operations after it
   __device__ __forceinline__ static double grid_point(uint32_t hi, uint32_t lo) {
     return __hiloint2double((int)(0x3ff00000u | (hi >> 12)),

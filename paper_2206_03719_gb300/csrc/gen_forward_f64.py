@@ -78,7 +78,7 @@ def main():
     with open(os.path.join(here, "forward_f64.h"), "w") as f:
         f.write("// forward_f64.h -- written by gen_forward_f64.py (40-digit mpmath); do not edit.\n"
                 "#pragma once\n\nnamespace lsmc {\n\n"
-                "constexpr int kQsOct = %d, kQsSeg = %d, kQsDeg = %d;  // octaves, segments, degree\n"
+                "constexpr int kQsOct = %d, kQsSeg = %d;  // octaves, segments\n"
                 "constexpr int kExpN = %d, kExpNLog2 = %d;\n"
                 "constexpr double kExpUnit = %.17e;  // kExpN / ln 2, as a pair\n"
                 "constexpr double kExpUnitLo = %.17e;\n"
@@ -91,7 +91,7 @@ def main():
                 "  float2 qp[3][kQsOct * kQsSeg];  // c_1, c_2, c_3 as pairs\n"
                 "  float qf[3][kQsOct * kQsSeg];   // c_4, c_5, c_6\n"
                 "  double exp2[kExpN];             // 2^(j / kExpN)\n"
-                "};\n\n" % ((OCT, SEG, DEG, EXPN, EXPN.bit_length() - 1, float(1 / L),
+                "};\n\n" % ((OCT, SEG, EXPN, EXPN.bit_length() - 1, float(1 / L),
                               float(1 / L - mp.mpf(float(1 / L))), float(L)) + pair(a1) + pair(a2) +
                              (float(a3),)))
         f.write("static __device__ const F64Tables kF64Tables = {\n    {\n")
