@@ -8,7 +8,9 @@ estimator and finite-difference Greeks) for the American-put book of
 
     python bench.py [--gpus N] [--steps K] [--warmup W] [--impl reference]
 
-Prints one JSON line.  Under torchrun (N > 1) every rank prices its own
+Prints one JSON line; the side measurements (other precisions, books, serving,
+bounds, ...), which make some 30 KB, go to bench_details.json beside this file
+with everything the line holds.  Under torchrun (N > 1) every rank prices its own
 replica of the workload on its own random stream (replicas only: the path
 needs no exchange) and rank 0 reports the units of all ranks over the
 slowest rank's time.
@@ -35,6 +37,7 @@ GOLDEN = os.path.join(_ROOT, "tests", "golden", "paper_fp64.json")
 GOLDEN_BOOK = os.path.join(_ROOT, "tests", "golden", "book_subset.json")
 GOLDEN_SERVING = os.path.join(_ROOT, "tests", "golden", "serving_subset.json")
 PEAKS = os.path.join(_ROOT, "MEASURED_PEAKS.json")
+DETAILS = os.path.join(_ROOT, "bench_details.json")
 # algorithmic work of the stepper (forward pass), counted from the formulas
 # of the scheme (a fused multiply-add counts 2 flops; elementary functions --
 # division, square root, exponential, logarithm -- counted apart, each one
@@ -725,6 +728,36 @@ def within_1e4_summary(line, acc, value):
             "outside_1e-4": out}
 
 
+# what the printed line holds, of the whole record and of its roofline (the
+# rest, and the side measurements, are in DETAILS): a record of 30 KB on
+# standard output came back cut where only its end is kept
+LINE_KEYS = ("metric", "value", "unit", "n_gpus", "steps", "warmup", "ms_per_step",
+             "higher_is_better", "scaling", "vs_baseline", "dtype", "data", "config",
+             "path_steps_per_s", "max_rel_err_vs_oracle", "accuracy_ok", "cpu_baseline", "e2e",
+             "gpu_launches", "clocks", "device_bytes")
+LINE_ROOFLINE = ("kernel", "bound", "achieved", "peak", "unit", "frac", "algorithmic_tflops",
+                 "traffic", "kernel_ms")
+
+
+def printed_line(record):
+    """The line to print for a whole record: a few kilobytes."""
+    line = {k: record[k] for k in LINE_KEYS if k in record}
+    if record.get("roofline"):
+        line["roofline"] = {k: record["roofline"].get(k) for k in LINE_ROOFLINE}
+    within = record.get("greeks_per_s_within_1e-4") or {}
+    line["greeks_per_s_within_1e-4"] = {k: within.get(k) for k in ("best", "best_greeks_per_s")}
+    line["details"] = os.path.basename(DETAILS)
+    return line
+
+
+def write_details(record):
+    try:
+        with open(DETAILS, "w") as f:
+            json.dump(record, f, indent=1)
+    except OSError as e:  # a read-only checkout loses the details, not the line
+        print("%s not written: %s" % (os.path.basename(DETAILS), e), file=sys.stderr)
+
+
 def run_cpu_full(wl, name):
     """The FP64 oracle once on the whole workload (every path, strike and
     revaluation) on all host cores: a full-size CPU baseline.  name
@@ -966,7 +999,8 @@ def main():
     if isinstance(ps, dict) and "mixed_large" in ps and "stepper_roofline" in ps["mixed_large"]:
         roofline["stepper"]["mixed_1048576"] = ps["mixed_large"]["stepper_roofline"]
     line["greeks_per_s_within_1e-4"] = within_1e4_summary(line, acc, value)
-    print(json.dumps(line), flush=True)
+    write_details(line)
+    print(json.dumps(printed_line(line)), flush=True)
     if dist is not None:
         dist.destroy_process_group()
 
