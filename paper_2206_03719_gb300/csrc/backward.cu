@@ -762,9 +762,15 @@ backward_kernel(BwdArgs a) {
                          ? V + ((ptrdiff_t)n - r0) * (ptrdiff_t)ld : nullptr;
 
     typename std::conditional<kFixed, FixedSums<BASIS>, Acc<Real, NA>>::type acc;
-    if constexpr (kFixed) acc.zero(s_fix[warp]);
-    else acc.zero();
+    if constexpr (kFixed) {
+      if (lane < kNSum) s_red[warp][lane] = 0.0;
+      acc.start(s_fix[warp]);
+    } else {
+      acc.zero();
+    }
     uint32_t n_itm = 0;  // in-the-money paths of this thread (monomial 1)
+    uint32_t n_out = 0;  // double: those whose sums are in s_red,
+    uint32_t n_set = 0;  // and those whose means are settled
     double euro = 0.0, sy = 0.0, sy2 = 0.0;
     uint32_t ties = 0;
 
@@ -1147,10 +1153,34 @@ backward_kernel(BwdArgs a) {
               item(have ? j0 + lane : j0, e, v, y);
               if (!acc.add(f, e, v, y, have && j0 != spilt, xK0, invTh)) break;
             }
-            if (j0 < full && acc.grow(s_fix[warp], held || j0 > 0, j0, full, !last, item, xK0, invTh))
-              spilt = j0;
+            if (j0 < full) {
+              const uint32_t added = n_itm + ((uint32_t)j0 >> 5);
+              acc.settle_mean(added - n_set);
+              n_set = added;
+              if (acc.grow(s_fix[warp], held || j0 > 0, j0, full, !last, item, xK0, invTh))
+                spilt = j0;
+            }
           }
           if (lane < full) n_itm += (uint32_t)(full - lane + 31) >> 5;
+          // the sums out of the lanes: added over the warp exactly, each
+          // converted by the lane that ends with it; at the end of the job and
+          // before a lane's integers can overflow
+          constexpr uint32_t kEvery = (kFixItems - 1) / PPT;
+          if (last || sb % kEvery == kEvery - 1) {
+            using Sums = FixedSums<BASIS>;
+            acc.settle_mean(n_itm - n_set);
+            long long ua[Sums::NU], ub[Sums::NU], oa, ob;
+            acc.units(ua, ub);
+            int i;
+            halving_units<Sums::NU, 16>(ua, ub, lane, 0, Sums::NU, oa, ob, i);
+            const uint32_t items = __reduce_add_sync(0xffffffffu, n_itm - n_out);
+            if (i >= 0)
+              s_red[warp][i < NM - 1 ? i + 1 : kSlotRhs + (i - (NM - 1))] +=
+                  Sums::value(i, oa, ob, s_fix[warp].scale, type == kPut);
+            if (lane == 0) s_red[warp][0] += (double)items;
+            n_out = n_set = n_itm;
+            acc.clear();
+          }
         } else {
           Real* t = acc.target();
           for (int j = lane; j < full; j += 32)
@@ -1189,20 +1219,12 @@ backward_kernel(BwdArgs a) {
       sy = warp_sum(sy);
       sy2 = warp_sum(sy2);
     } else if constexpr (!kSingle) {
-      // double: the fixed-point units reduced exactly over the lanes, each
-      // converted by the lane that ends with it
-      using Sums = FixedSums<BASIS>;
-      long long ua[Sums::NU], ub[Sums::NU], oa, ob;
-      acc.units(ua, ub);
-      int i;
-      halving_units<Sums::NU, 16>(ua, ub, lane, 0, Sums::NU, oa, ob, i);
-      const uint32_t items = __reduce_add_sync(0xffffffffu, n_itm);
-      auto slot = [](int u) { return u < NM - 1 ? u + 1 : kSlotRhs + (u - (NM - 1)); };
-      if (i >= 0) s_red[warp][slot(i)] = Sums::value(i, oa, ob, s_fix[warp].scale, type == kPut);
-      if (lane == 0) s_red[warp][0] = (double)items;
+      // double: the fixed-point sums are in s_red already
       if (s_fix[warp].spilled) {
         __syncwarp();
-        if (lane < Sums::NU) s_red[warp][slot(lane)] += s_fix[warp].spill[lane];
+        if (lane < FixedSums<BASIS>::NU)
+          s_red[warp][lane < NM - 1 ? lane + 1 : kSlotRhs + (lane - (NM - 1))] +=
+              s_fix[warp].spill[lane];
       }
     } else {
       // rows per pass: as many as the warp's moment buffers hold

@@ -5,26 +5,28 @@
 // clocks a warp, a 32 x 32 -> 64-bit integer multiply-add for 0.66.  The 21
 // sums of an in-the-money path took 25 FP64 operations (425 clocks per 32
 // paths), four fifths of the backward pass's FP64 work; here 2 FP64
-// operations, 61 integer multiply-adds and about 120 other integer
+// operations, 47 integer multiply-adds and about 110 other integer
 // instructions do it.
 // (The FP64 matrix instruction m8n8k4 runs at 3.6 times the FP64 rate, 36
 // clocks, but an 8 x 8 tile holds the 21 sums once: 377 clocks for 32 paths.)
 //
 // Format.  A value q (x, w or the cash flow y, formed in double) is the
-// integer round(q 2^F), |.| < 2^54, from its mantissa by shifts, split into
+// integer round(q 2^F), |.| < 2^56, from its mantissa by shifts, split into
 // limbs h 2^28 + l, |l| <= 2^27.  The squares and the product x w keep the
-// format (round(X X 2^-54), ...).  A product of two values adds h h' to one
-// 64-bit sum and h l' + l h' + (l l' 2^-28) to another, l l' from 14 bits of
-// each; 256 paths a lane (the largest job) stay below 2^63.  The sums of 32
-// lanes are added and converted without a rounding before the last.  (Without
-// l l', which is of mean 2^54 / 3 in the squares of x^2 and w^2, the sums of
-// x^4 and w^4 came out 1e-14 to 1e-13 low: 39.4 against 41.0 ms with it for
-// the book of 131,072 x 252 x 55.)  Over maturities from a day to a year,
-// volatilities of variance from 0.001 to 0.3 and 40 to 2,000 paths the fits
-// are as near the exact ones as those of double sums
+// format (round(X X 2^-56), ...).  A product of two values adds h h' to one
+// 64-bit sum and h l' + l h' to another; l l' is below 2^-58 of the range's
+// product and of mean zero, but for the squares of x^2 and w^2, which get its
+// mean.  A lane sums 64 paths at most before its sums are taken out, added over
+// the warp without a rounding and converted.  (With 54 bits, which 256 paths, a
+// whole job, do not overflow, the part left out is 16 times larger and its mean
+// put the sums of x^4 and w^4 1e-14 to 1e-13 too low; with the products of the
+// low limbs summed as well the book of 131,072 x 252 x 55 took 41.3 ms, against
+// 39.6 like this.)  Over maturities from a day to a year, volatilities of variance
+// from 0.001 to 0.3 and 40 to 2,000 paths the sums are as near the exact ones
+// as those in double, the fits a little nearer
 // (tests/test_fixed_moments_host.py runs this code on the host).
 //
-// Range.  2^(54 - F) is the smallest power of two above the largest |q| that
+// Range.  2^(56 - F) is the smallest power of two above the largest |q| that
 // the warp has summed in its job, for x, w and y each (for y, of which only
 // first powers are summed, with two bits to spare while more paths may come).
 // It is taken from the first list of paths; when a later path lies beyond it,
@@ -49,7 +51,10 @@
 namespace lsmc {
 namespace {
 
-constexpr int kFixBits = 54;  // |integer| < 2^54
+constexpr int kFixBits = 56;  // |integer| < 2^56
+// Paths a lane may sum before its sums are taken out:
+// h h' below 2^56 each.
+constexpr int kFixItems = 64;
 // Largest ranges: x and w < 2^kFixTopXW, cash flows < 2^kFixTopY (values
 // beyond, infinities and NaN are summed in double).  The scales start at ranges
 // 2^-kFixTopXW and 2^-kFixTopY.  With these every scale of a sum is a normal
@@ -80,9 +85,6 @@ __device__ __forceinline__ unsigned long long shr_clamped(unsigned long long v, 
 struct Limbs {
   int h, l;
   Limbs() = default;
-  // l 2^-14, for the product of two low limbs in units of 2^28 (14 bits of
-  // each: within 2^-13 of it)
-  __device__ __forceinline__ int top() const { return l >> 14; }
   // the limbs of v
   __device__ __forceinline__ explicit Limbs(long long v) {
     const long long r = v + (1ll << 27);
@@ -93,14 +95,15 @@ struct Limbs {
 
 // The limbs of |q| 2^F, from the mantissa m and the exponent field e of q
 // (|q| = m 2^(e - 1075)); hi: the high word of |q|.  bad: |q| outside the
-// range, e > 1076 - F (then the limbs mean nothing).
+// range, e > kFixTop - F (then the limbs mean nothing).
+constexpr int kFixTop = 1022 + kFixBits;
 __device__ __forceinline__ Limbs fix_magnitude(int hi, int lo, int F, bool& bad) {
-  // m shifted left by 3 and right by n: twice the integer, the last bit rounding
-  const int n = 1077 - F - (hi >> 20);
+  // m shifted left by 5 and right by n: twice the integer, the last bit rounding
+  const int n = kFixTop + 1 - F - (hi >> 20);
   bad = bad || n < 1;
   const uint32_t mh = ((uint32_t)hi & 0xfffffu) | 0x100000u;
-  const unsigned long long m = ((unsigned long long)__funnelshift_l((uint32_t)lo, mh, 3) << 32) |
-                               ((uint32_t)lo << 3);
+  const unsigned long long m = ((unsigned long long)__funnelshift_l((uint32_t)lo, mh, 5) << 32) |
+                               ((uint32_t)lo << 5);
   // zero for shifts beyond 63 (small values, and the bad ones)
   const unsigned long long t = shr_clamped(m, n) + (1ull + (1ull << 28));
   Limbs r;
@@ -120,7 +123,7 @@ __device__ __forceinline__ Limbs fix_signed(double q, int F, bool& bad) {
 // The sums of a basis as units, in slot order without the count: a sum of
 // products (hh 2^56 + hl 2^28) 2^-E or a plain sum of integers.  Packed per
 // unit: powers of x, w, y (4 bits each), the number of operands that are
-// themselves products (each drops 2^54), and whether it is a plain sum.
+// themselves products (each drops 2^kFixBits), and whether it is a plain sum.
 constexpr uint32_t fix_unit(int a, int b, int c, int prods, int plain) {
   return (uint32_t)(a | b << 4 | c << 8 | prods << 12 | plain << 16);
 }
@@ -156,14 +159,14 @@ __device__ __forceinline__ long long wide(int a, int b, long long c) {
   return (long long)a * b + c;
 #endif
 }
-// round(A B 2^-54)
+// round(A B 2^-56)
 __device__ __forceinline__ long long fix_product(const Limbs& a, const Limbs& b) {
-  return wide(4 * a.h, b.h, wide(a.l, b.h, wide(a.h, b.l, 1ll << 25)) >> 26);
+  return wide(a.h, b.h, wide(a.l, b.h, wide(a.h, b.l, 1ll << 27)) >> 28);
 }
 // the same for a square; l l, of mean 2^54 / 3, is not formed: its mean is
 // added instead
 __device__ __forceinline__ long long fix_square(const Limbs& a) {
-  return wide(4 * a.h, a.h, wide(a.h + a.h, a.l, (1ll << 25) + (1ll << 26) / 3) >> 26);
+  return wide(a.h, a.h, wide(a.h + a.h, a.l, (1ll << 27) + (1ll << 26) / 3) >> 28);
 }
 
 // What a warp's lanes share, in shared memory: the scales of the sums, and the
@@ -189,10 +192,13 @@ template <int BASIS> struct FixedSums {
   __device__ __forceinline__ static uint32_t unit(int u) {
     return kV ? kFixUnitsSV2[u] : kFixUnitsS2[u];
   }
-  // called by the whole warp
-  __device__ __forceinline__ void zero(FixWarp& ws) {
+  __device__ __forceinline__ void clear() {
 #pragma unroll
     for (int i = 0; i < NU; ++i) hh[i] = hl[i] = 0;
+  }
+  // called by the whole warp, once per job
+  __device__ __forceinline__ void start(FixWarp& ws) {
+    clear();
     const int lane = threadIdx.x & 31;
     if (lane < NU) ws.spill[lane] = 0.0;
     if (lane == 0) {
@@ -206,11 +212,11 @@ template <int BASIS> struct FixedSums {
   }
   __device__ __forceinline__ void product(int i, const Limbs& a, const Limbs& b) {
     hh[i] = wide(a.h, b.h, hh[i]);
-    hl[i] = wide(a.l, b.h, wide(a.h, b.l, wide(a.top(), b.top(), hl[i])));
+    hl[i] = wide(a.l, b.h, wide(a.h, b.l, hl[i]));
   }
   __device__ __forceinline__ void square(int i, const Limbs& a) {
     hh[i] = wide(a.h, a.h, hh[i]);
-    hl[i] = wide(a.h + a.h, a.l, wide(a.top(), a.top(), hl[i]));
+    hl[i] = wide(a.h + a.h, a.l, hl[i]);
   }
   // The sums from scales f to scales n <= f, in steps that divide no unit by
   // more than 2^28: a plain sum is rounded, of the others hl keeps what hh
@@ -282,13 +288,20 @@ template <int BASIS> struct FixedSums {
     }
     return true;
   }
+  // Adds to the squares the mean of the l l left out of `items` of this lane's
+  // paths, at the scales they were summed at.
+  __device__ __forceinline__ void settle_mean(uint32_t items) {
+    hl[3] += (long long)items * ((1 << 26) / 3);
+    if (kV) hl[kV ? 13 : 0] += (long long)items * ((1 << 26) / 3);
+  }
   // Takes the scales (and the sums, if there are any) to what covers every path
   // from j0 on of a list of `full`; or, where they do already and add() refused
   // paths [j0, j0 + 32), sums this chunk's paths beyond the largest range in
   // double, a monomial per lane, and returns true for their lanes.
   // item(j, e, v, z) gives a path's values.  more: other lists may follow; y,
   // of which only first powers are summed, then gets two bits above its
-  // largest value.  Called by the whole warp.
+  // largest value.  After settle_mean of all paths added; called by the whole
+  // warp.
   template <typename Item>
   __device__ __forceinline__ bool grow(FixWarp& ws, bool any, int j0, int full, bool more,
                                        const Item& item, double xK, double invTh) {
@@ -311,10 +324,10 @@ template <int BASIS> struct FixedSums {
     ex = __reduce_max_sync(0xffffffffu, ex);
     if (kV) ew = __reduce_max_sync(0xffffffffu, ew);
     ey = __reduce_max_sync(0xffffffffu, ey);
-    FixScale n;
-    n.x = min(f.x, 1076 - ex);
-    n.w = kV ? min(f.w, 1076 - ew) : f.w;
-    n.y = ey > 1076 - f.y ? 1076 - ey - (more ? 2 : 0) : f.y;
+    FixScale n = f;
+    n.x = min(f.x, kFixTop - ex);
+    if (kV) n.w = min(f.w, kFixTop - ew);
+    n.y = ey > kFixTop - f.y ? kFixTop - ey - (more ? 2 : 0) : f.y;
     if (n.x != f.x || n.w != f.w || n.y != f.y) {
       if (any) rescale(f, n);
       __syncwarp();
@@ -325,8 +338,9 @@ template <int BASIS> struct FixedSums {
     double e, v, z;
     item(min(j0 + lane, full - 1), e, v, z);
     const double xd = fma(e, xK, -1.0), wd = kV ? fma(v, invTh, -1.0) : 0.0;
-    const bool bad = j0 + lane < full && (exponent(xd) > 1076 - f.x || exponent(wd) > 1076 - f.w ||
-                                          exponent(z) > 1076 - f.y);
+    const bool bad = j0 + lane < full && (exponent(xd) > kFixTop - f.x ||
+                                          exponent(wd) > kFixTop - f.w ||
+                                          exponent(z) > kFixTop - f.y);
     double p = 0.0;
     const uint32_t u = unit(lane < NU ? lane : 0);
     unsigned m = __ballot_sync(0xffffffffu, bad);
@@ -355,7 +369,7 @@ template <int BASIS> struct FixedSums {
       b[i] = (h & kMask) << 28 | (is_plain(i) ? 0 : hl[i] & kMask);
     }
   }
-  // neg: x is negative (puts)
+  // a unit added over the lanes; neg: x is negative (puts)
   __device__ __forceinline__ static double value(int u, long long a, long long b,
                                                  const FixScale& f, bool neg) {
     const uint32_t t = unit(u);

@@ -20,7 +20,8 @@ void fixed_sums_t(int n, int per, const double* e, const double* v, const double
     for (int w0 = 0; w0 < n; w0 += per) {
       const int m = std::min(per, n - w0);
       Sums acc;
-      acc.zero(ws);
+      acc.start(ws);
+      uint32_t settled = 0;  // of this lane's paths
       auto item = [&](int j, double& ej, double& vj, double& zj) {
         ej = e[w0 + j];
         vj = v[w0 + j];
@@ -41,12 +42,15 @@ void fixed_sums_t(int n, int per, const double* e, const double* v, const double
             spilt = false;
             any = true;
           } else {
+            acc.settle_mean((uint32_t)j0 / 32 - settled);
+            settled = (uint32_t)j0 / 32;
             spilt = acc.grow(ws, any, j0, full, more, item, xK, invTh);
           }
         }
       }
       long long a[Sums::NU], b[Sums::NU], oa, ob;
       int i;
+      acc.settle_mean((uint32_t)(m - lane + 31) / 32 * (lane < m) - settled);
       acc.units(a, b);
       halving_units<Sums::NU, 16>(a, b, lane, 0, Sums::NU, oa, ob, i);
       if (i >= 0) part[i] = Sums::value(i, oa, ob, ws.scale, neg != 0);

@@ -1,14 +1,15 @@
-// A warp on the host: 32 threads and the CUDA intrinsics that fixed_moments.cuh
-// uses, so that the header's own arithmetic can be run and checked on the CPU.
+// A warp on the host: 32 lanes as coroutines that take turns at every warp
+// operation, and the CUDA intrinsics that fixed_moments.cuh uses, so that the
+// header's own arithmetic can be run and checked on the CPU.
 #pragma once
 
+#include <ucontext.h>
+
 #include <algorithm>
-#include <barrier>
 #include <cmath>
 #include <cstdint>
 #include <cstring>
 #include <functional>
-#include <thread>
 #include <vector>
 
 #define __device__
@@ -18,9 +19,31 @@
 using std::max;
 using std::min;
 
-static thread_local struct { unsigned x; } threadIdx;
-static std::barrier<> warp_barrier(32);
+static struct { unsigned x; } threadIdx;
+static ucontext_t warp_lane[32], warp_caller;
+static bool warp_done[32];
+static const std::function<void(int)>* warp_main;
 static long long warp_slot[32];
+
+// The next lane's turn: a lane runs on when every other has come as far.
+static void next_lane() {
+  const int me = threadIdx.x;
+  for (int k = 1; k <= 32; ++k) {
+    const int i = (me + k) & 31;
+    if (!warp_done[i]) {
+      threadIdx.x = i;
+      if (i != me) swapcontext(&warp_lane[me], &warp_lane[i]);
+      return;
+    }
+  }
+  setcontext(&warp_caller);  // all done
+}
+static void lane_entry() {
+  const int me = threadIdx.x;
+  (*warp_main)(me);
+  warp_done[me] = true;
+  next_lane();
+}
 
 template <typename T> static T lane_value(int lane) {
   T v;
@@ -30,9 +53,9 @@ template <typename T> static T lane_value(int lane) {
 // every lane's value, combined by f after all have written theirs
 template <typename T, typename F> static auto warp_exchange(T v, F f) {
   memcpy(&warp_slot[threadIdx.x], &v, sizeof(T));
-  warp_barrier.arrive_and_wait();
+  next_lane();
   auto r = f();
-  warp_barrier.arrive_and_wait();
+  next_lane();
   return r;
 }
 static inline unsigned __ballot_sync(unsigned, bool p) {
@@ -43,7 +66,7 @@ static inline unsigned __ballot_sync(unsigned, bool p) {
   });
 }
 static inline bool __any_sync(unsigned m, bool p) { return __ballot_sync(m, p) != 0; }
-static inline void __syncwarp() { warp_barrier.arrive_and_wait(); }
+static inline void __syncwarp() { next_lane(); }
 template <typename T> static T __shfl_sync(unsigned, T v, int src) {
   return warp_exchange<T>(v, [=] { return lane_value<T>(src & 31); });
 }
@@ -77,11 +100,17 @@ static inline int __ffs(unsigned m) { return __builtin_ffs((int)m); }
 static inline int __mulhi(int a, int b) { return (int)(((long long)a * b) >> 32); }
 
 static inline void run_warp(const std::function<void(int)>& lane_main) {
-  std::vector<std::thread> t;
-  for (int i = 0; i < 32; ++i)
-    t.emplace_back([&, i] {
-      threadIdx.x = i;
-      lane_main(i);
-    });
-  for (auto& x : t) x.join();
+  constexpr size_t kStack = 1 << 18;
+  std::vector<char> stacks(32 * kStack);
+  warp_main = &lane_main;
+  for (int i = 0; i < 32; ++i) {
+    warp_done[i] = false;
+    getcontext(&warp_lane[i]);
+    warp_lane[i].uc_stack.ss_sp = stacks.data() + i * kStack;
+    warp_lane[i].uc_stack.ss_size = kStack;
+    warp_lane[i].uc_link = nullptr;
+    makecontext(&warp_lane[i], lane_entry, 0);
+  }
+  threadIdx.x = 0;
+  swapcontext(&warp_caller, &warp_lane[0]);
 }

@@ -1,5 +1,5 @@
 """The double-precision regressions' fixed-point moment sums on the CPU: the
-header's own code (fixed_moments.cuh) on a warp of host threads, against exact
+header's own code (fixed_moments.cuh) on a warp of host coroutines, against exact
 rational sums, over maturities, volatilities and distances of v0 from theta."""
 import ctypes
 import os
@@ -17,9 +17,9 @@ CSRC = os.path.join(os.path.dirname(HERE), "paper_2206_03719_gb300", "csrc")
 @pytest.fixture(scope="module")
 def lib(tmp_path_factory):
     so = str(tmp_path_factory.mktemp("fixed") / "fixed_moments_host.so")
-    subprocess.run(["g++", "-std=c++20", "-O2", "-ffp-contract=off", "-shared", "-fPIC",
+    subprocess.run(["g++", "-std=c++17", "-O2", "-ffp-contract=off", "-shared", "-fPIC",
                     "-I" + HERE, "-I" + CSRC, os.path.join(HERE, "fixed_moments_host.cpp"),
-                    "-o", so, "-lpthread"], check=True)
+                    "-o", so], check=True)
     return ctypes.CDLL(so)
 
 
@@ -155,6 +155,23 @@ def test_scales_follow_values_that_grow_and_any_units(lib, basis):
         s = _sums(lib, "fixed", basis, 640, e * f, v, y * f, 1.0 / (K * f), 1.0 / theta, False)
         for u, t, b in zip(R.UNITS[basis], s, base):
             assert t == (b * f if u[2] else b), (u, k)
+
+
+@pytest.mark.parametrize("basis", ["s2", "sv2"])
+@pytest.mark.parametrize("n", [61 * 32, 63 * 32 + 1])
+def test_largest_sums(lib, basis, n):
+    # as many paths as a lane may sum, each at the top of its range: no sum
+    # overflows (with equal values the part left out of the squares is at most
+    # 2^-58 of them, below the bound)
+    K, theta = 100.0, 0.04
+    e, v = np.full(n, K * 2.0**-50), np.full(n, theta * (9.0 - 2.0**-49))
+    y = np.full(n, 128.0 * (1.0 - 2.0**-53))
+    s = _sums(lib, "fixed", basis, n, e, v, y, 1.0 / K, 1.0 / theta, True)
+    x, w = R.feature(e, 1.0 / K), R.feature(v, 1.0 / theta)
+    assert 1 - 2.0**-40 < -x[0] < 1 and 8 - 2.0**-40 < w[0] < 8
+    m, a = R.moments(x, w, y, basis), R.moments(np.abs(x), np.abs(w), y, basis)
+    for u, t in zip(R.UNITS[basis], s):
+        assert abs(float(R.Fraction(float(t)) - m[u])) <= 4 * R.EPS * float(a[u]), (u, t)
 
 
 @pytest.mark.parametrize("basis", ["s2", "sv2"])

@@ -119,6 +119,29 @@ def test_dates_of_very_different_spread(torch, basis, narrow_S, narrow_V):
     _check(torch, S, V, H, 100.0, 1.0, True, basis, "spread")
 
 
+@pytest.mark.parametrize("option", ["put", "call"])
+@pytest.mark.parametrize("basis", ["s2", "sv2"])
+def test_jobs_whose_sums_are_taken_out_more_than_once(torch, basis, option):
+    # more paths a lane than its integers hold (from 15 sub-tiles of 4 paths,
+    # 31 of 2), deep in the money so that every path is summed: the prices of
+    # jobs of one sub-tile (no decision lies within 1e-12 of its threshold)
+    from paper_2206_03719_gb300 import api, workloads
+    K = 190.0 if option == "put" else 30.0
+    wl = workloads.SMALL_FP64.replace(n_paths=40013, n_steps=5, basis=basis, option=option,
+                                      greeks=("delta",), strikes=[K, 100.0],
+                                      model=dict(H, q=0.04))
+    rows = {}
+    with api.Context(workspace_bytes=1 << 30) as ctx:
+        for shape in ((1, 4), (15, 4), (16, 4), (32, 2), (64, 4)):
+            ctx.set_backward_shape(*shape)
+            rows[shape] = ctx.price(wl)
+    for shape, got in rows.items():
+        for g, r in zip(got, rows[1, 4]):
+            for k in ("price", "price_se", "delta"):
+                assert abs(g[k] - r[k]) <= 1e-12 * max(abs(r[k]), 1e-3), (shape, k, g[k], r[k])
+            assert g["n_singular_solves"] == r["n_singular_solves"]
+
+
 @pytest.mark.parametrize("basis", ["s2", "sv2"])
 def test_call_deep_in_the_money(torch, basis):
     model = dict(H, S0=600.0, q=0.05)
