@@ -16,7 +16,7 @@
 // format (round(X X 2^-56), ...).  A product of two values adds h h' to one
 // 64-bit sum and h l' + l h' to another; l l' is below 2^-58 of the range's
 // product and of mean zero, but for the squares of x^2 and w^2, which get its
-// mean.  A lane sums 64 paths at most before its sums are taken out, added over
+// mean.  A lane sums 126 paths at most before its sums are taken out, added over
 // the warp without a rounding and converted.  (With 54 bits, which 256 paths, a
 // whole job, do not overflow, the part left out is 16 times larger and its mean
 // put the sums of x^4 and w^4 1e-14 to 1e-13 too low; with the products of the
@@ -52,9 +52,10 @@ namespace lsmc {
 namespace {
 
 constexpr int kFixBits = 56;  // |integer| < 2^56
-// Paths a lane may sum before its sums are taken out:
-// h h' below 2^56 each.
-constexpr int kFixItems = 64;
+// Paths a lane may sum before its sums are taken out: h h', h l' + l h' and the
+// values themselves are at most 2^56 each, so 126 of them, and what shifts and
+// means add, stay below 2^63.
+constexpr int kFixItems = 126;
 // Largest ranges: x and w < 2^kFixTopXW, cash flows < 2^kFixTopY (values
 // beyond, infinities and NaN are summed in double).  The scales start at ranges
 // 2^-kFixTopXW and 2^-kFixTopY.  With these every scale of a sum is a normal

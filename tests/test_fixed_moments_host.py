@@ -158,7 +158,7 @@ def test_scales_follow_values_that_grow_and_any_units(lib, basis):
 
 
 @pytest.mark.parametrize("basis", ["s2", "sv2"])
-@pytest.mark.parametrize("n", [61 * 32, 63 * 32 + 1])
+@pytest.mark.parametrize("n", [61 * 32, 125 * 32 + 1, 126 * 32])
 def test_largest_sums(lib, basis, n):
     # as many paths as a lane may sum, each at the top of its range: no sum
     # overflows (with equal values the part left out of the squares is at most

@@ -122,8 +122,8 @@ def test_dates_of_very_different_spread(torch, basis, narrow_S, narrow_V):
 @pytest.mark.parametrize("option", ["put", "call"])
 @pytest.mark.parametrize("basis", ["s2", "sv2"])
 def test_jobs_whose_sums_are_taken_out_more_than_once(torch, basis, option):
-    # more paths a lane than its integers hold (from 15 sub-tiles of 4 paths,
-    # 31 of 2), deep in the money so that every path is summed: the prices of
+    # more paths a lane than its integers hold (beyond 31 sub-tiles of 4 paths,
+    # 62 of 2), deep in the money so that every path is summed: the prices of
     # jobs of one sub-tile (no decision lies within 1e-12 of its threshold)
     from paper_2206_03719_gb300 import api, workloads
     K = 190.0 if option == "put" else 30.0
@@ -132,7 +132,7 @@ def test_jobs_whose_sums_are_taken_out_more_than_once(torch, basis, option):
                                       model=dict(H, q=0.04))
     rows = {}
     with api.Context(workspace_bytes=1 << 30) as ctx:
-        for shape in ((1, 4), (15, 4), (16, 4), (32, 2), (64, 4)):
+        for shape in ((1, 4), (15, 4), (16, 4), (31, 4), (32, 4), (63, 2), (64, 4)):
             ctx.set_backward_shape(*shape)
             rows[shape] = ctx.price(wl)
     for shape, got in rows.items():
