@@ -180,7 +180,8 @@ struct JobInfo {
 // each, atomics one after the other, the solve on one thread -- now run over
 // the lanes, overlap or sit beside the solve: 35.9 -> 32.0 ms (float pairs 32.3
 // -> 31.3, single precision 83.5 -> 80.1 at 1,048,576 paths; jobs of one
-// sub-tile of 128 paths 152 -> 108).
+// sub-tile of 128 paths 152 -> 108).  At 12 sub-tiles 27.4 ms; 29.5 since each
+// warp scales its sums by its own paths (fixed_moments.cuh).
 //
 // Threads per CTA of the backward pass and resident CTAs per SM: 64 x 8 for
 // double (shorter barriers around the FP64 pipe's work: the FP64 backward of
