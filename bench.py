@@ -73,9 +73,10 @@ BWD_FLOPS_ITM = 40 + 15
 # cash flows grow in proportion).  Instruction issue bounds the kernel: its
 # moment sums are integer multiply-adds and its exercise test mostly runs in
 # single precision, so the double-precision pipe is a quarter busy.  Valid only
-# for the source (null once the code of backward.cu or fixed_moments.cuh changes,
-# capture_source_hash) and the paths per lane it was taken with; the bytes only for its sub-tiles per job
-# too (the instructions differ by 4% between 8 and 12).
+# for the source (null once the code of backward.cu or fixed_moments.cuh
+# changes, capture_source_hash) and the paths per lane it was taken with; the
+# bytes only for its sub-tiles per job too (the instructions differ by 4%
+# between 8 and 12).
 BWD_CAPTURE = {"inst_per_path_date": 15091452257 * 32 / (98304 * 252 * 55),
                "bytes": (3.090159872e9 + 0.330531840e9) * 131072 / 98304,
                "shape": (12, 4),
